@@ -83,7 +83,10 @@ typedef enum {
 } paw_status;
 
 typedef enum {
-  PAW_FP64 = 0,  /* every step in FP64: the plain method                      */
+  PAW_FP64 = 0,  /* FP64 data and FP64-level accuracy in every step: the plain */
+                 /* method (the local cell contractions run in 59-bit fixed    */
+                 /* point per cell and vector, with errors no larger than      */
+                 /* those of FP64 sums)                                        */
   PAW_FP32 = 1,  /* filter bracket in FP32 storage and FP32 FMA arithmetic     */
   PAW_TF32 = 2,  /* FP32 storage; cell products and projector contractions   */
                  /* on tcgen05 tensor cores (TF32 operands, FP32 accumulation */

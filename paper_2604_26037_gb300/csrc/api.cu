@@ -285,7 +285,7 @@ static void residual_block(paw_context *c, const double *X, int ldx, const doubl
   // at k != 0 the Bloch term -i B of Eq. hij on the split block [Re | Im]
   {
     PhaseScope ps(c, 0, s);
-    local_sf(c, X, ldx, Y, ldy, ncols, 1.0, 1.0, 1.0, c->kmass, negLam_dev, s, pair);
+    local_sf(c, X, ldx, Y, ldy, ncols, 1.0, 1.0, 1.0, c->kmass, negLam_dev, s);
     if (c->kc) {
       bloch_sf(c, X + ncols / 2, ldx, Y, ldy, ncols / 2, 1.0, s);
       bloch_sf(c, X, ldx, Y + ncols / 2, ldy, ncols / 2, -1.0, s);
@@ -1095,7 +1095,7 @@ paw_status paw_destroy(paw_handle c) {
                     &c->Gfull32, &c->apair_off, &c->apair, &c->nltc.projB, &c->nltc.projBs, &c->nltc.expB, &c->nltc.mdo, &c->nltc.odof, &c->status_dev, &c->proj_ext_dev, &c->own_ngrp,
                     &c->own_lg, &c->own_sidx, &c->own_cnt, &c->Bk64, &c->Bk32, &c->tc_bk_tf32.He,
                     &c->tc_bk_bf16.He, &c->ws_cx, &c->ws_cy,
-                    &c->nltc.eoff, &c->ownPx2, &c->wVx2,
+                    &c->nltc.eoff, &c->ownPx2, &c->wVs,
                     &c->scr_main.partial, &c->scr_main.pp, &c->scr_main.W2, &c->scr_main.Wx2,
                     &c->scr_side.partial, &c->scr_side.pp, &c->scr_side.W2, &c->scr_side.Wx2,
                     &c->ws_Y0p[0], &c->ws_Y0p[1], &c->ws_cxp[0], &c->ws_cxp[1], &c->ws_cyp[0], &c->ws_cyp[1], &c->ws_lamp[0], &c->ws_lamp[1], &c->ws_cfp[0], &c->ws_cfp[1]};

@@ -182,10 +182,9 @@ struct paw_context {
   pawfe::DevBuf Me64, Me32, K64;              // nc*nc
   pawfe::DevBuf Nq64, wq64;                   // nq*nc, nq
   pawfe::DevBuf Vq;                           // ncells*nq
-  pawfe::DevBuf wV;                           // ncells*nq: w_q detJ V_q (sum-factorised V^e)
+  pawfe::DevBuf wV;                           // ncells*nq: w_q detJ V_q in fixed point (sum-factorised V^e)
   int wV_valid = 0;
-  int wVx2_valid = 0;                          // wVx2 = wV as pairs of FP32 numbers
-  pawfe::DevBuf wVx2;
+  pawfe::DevBuf wVs;                          // ncells: exponents of wV's fixed-point numbers
   pawfe::TcMats tc_tf32, tc_bf16;
   pawfe::TcMats tc_bk_tf32, tc_bk_bf16;       // tcgen05 images of B^e (one shared matrix)
   pawfe::NlTcMats nltc;
@@ -331,11 +330,10 @@ void nl_residual_pair(paw_context *c, const double *X, int ldx, int ncols, const
 // expansion with the output stage of mode (EXP_ADD / EXP_SINV / EXP_RECURRENCE)
 struct ExpArgs;
 void nltc_expand(paw_context *c, int mode, const ExpArgs &A, const float *W1, const float *W2, cudaStream_t s);
-// FP64 sum-factorised local operator (sumfac.cu):
+// sum-factorised local operator on FP64 data (sumfac.cu):
 // Y += alpha * (cK K^e + cV V^e + (cM + cMcol[j]) M^e) X, cell by cell with assembly;
-// pair32: the contractions in pair-of-FP32 arithmetic (f32x2.cuh), X and Y FP64
 void local_sf(paw_context *c, const double *X, int ldx, double *Y, int ldy, int ncols, double alpha,
-              double cK, double cV, double cM, const double *cMcol, cudaStream_t s, bool pair32 = false);
+              double cK, double cV, double cM, const double *cMcol, cudaStream_t s);
 // FP64 sum-factorised Bloch term: Y += alpha * B X, B = sum_d k_d G_d cell by cell
 // (G_d the skew cell form of int N_I dN_J/dx_d, Eq. hij), with assembly
 void bloch_sf(paw_context *c, const double *X, int ldx, double *Y, int ldy, int ncols, double alpha,
