@@ -260,19 +260,14 @@ static void merge_cplx(paw_context *c, const T *Xs, int n, T *Z, int ldz, cudaSt
   PAW_LAUNCH_CHECK("k_merge_cplx");
 }
 
-// Y = H X - S X Lambda in FP64 (Algorithm 2 step 2), or in pair-of-FP32 arithmetic
-// with FP64 data when options.y0_pair32 is set
+// Y = H X - S X Lambda in FP64 (Algorithm 2 step 2)
 static void residual_block(paw_context *c, const double *X, int ldx, const double *negLam_dev,
                            double *Y, int ldy, int ncols, cudaStream_t s) {
   zero_block<double>(Y, c->ndof, ncols, ldy, s);
-  const bool pair = c->opts.y0_pair32 != 0;   // pair-of-FP32 arithmetic (k = 0 only, checked at create)
   // both parts add into Y (the local part first: with the nonlocal part first beside a
   // loop, the mid filter call measured 293 instead of 288 ms)
   auto nonlocal = [&]() {
-    if (c->nown_pairs > 0 && pair) {
-      PhaseScope ps(c, 4, s);
-      nl_residual_pair(c, X, ldx, ncols, c->DH64.as<double>(), c->DS64.as<double>(), negLam_dev, Y, ldy, s);
-    } else if (c->nown_pairs > 0) {
+    if (c->nown_pairs > 0) {
       PhaseScope ps(c, 4, s);
       // sum_a P^a (D_H^a - lambda_j dS^a) P^a^T x_j: one projection, one expansion
       c->scr->W2.ensure(sizeof(double) * (size_t)c->natoms * c->npad * ncols, &c->dev_bytes);
@@ -905,8 +900,7 @@ static void apply_any(paw_context *c, paw_precision prec, int which, const void 
                       int ncols, cudaStream_t s) {
   if (prec == PAW_F32X2) {
     PAW_REQUIRE(!c->kc, PAW_ERR_UNSUPPORTED, "PAW_F32X2 is implemented for real vectors (k = 0)");
-    op_pair(c, which, (const double *)X, ldx, (double *)Y, ldy, ncols, s);
-    return;
+    prec = PAW_FP64;   // the FP64 kernels run on the integer pipes and tensor cores and are the faster form
   }
   if (c->kc) {
     if (prec == PAW_FP64)
@@ -1086,18 +1080,18 @@ paw_status paw_destroy(paw_handle c) {
   cudaDeviceSynchronize();
   DevBuf *bufs[] = {&c->cell_dofs, &c->md_inv64, &c->md_inv32, &c->He64, &c->He32, &c->Me64, &c->Me32,
                     &c->K64, &c->Nq64, &c->wq64, &c->Vq, &c->tc_tf32.He, &c->tc_tf32.Me, &c->tc_bf16.He,
-                    &c->tc_bf16.Me, &c->ent_dof, &c->P64, &c->P32, &c->own_off, &c->own_atom, &c->ownP64,
+                    &c->tc_bf16.Me, &c->ent_dof, &c->P64, &c->P32, &c->own_off, &c->own_atom, &c->own_proj_dg, &c->own_exp_dg, &c->own_sP, &c->own_mask,
                     &c->ownP32,
                     &c->DH64, &c->DS64, &c->DSinv64, &c->ws_W, &c->ws_RX,
                     &c->ws_RY, &c->ws_T, &c->ws_Y0f, &c->ws_colscale, &c->ws_red, &c->ws_vec,
                     &c->ws_HX, &c->ws_SX, &c->ws_Hp, &c->ws_Sp, &c->ws_eig, &c->ws_solver, &c->ws_info,
                     &c->ws_rot, &c->ws_gram, &c->ws_cg, &c->wV, &c->ws_Y0lo, &c->gnb_off, &c->gnb_atom, &c->Gfull, &c->Fsh32, &c->DSinv32,
                     &c->Gfull32, &c->apair_off, &c->apair, &c->nltc.projB, &c->nltc.projBs, &c->nltc.expB, &c->nltc.mdo, &c->nltc.odof, &c->status_dev, &c->proj_ext_dev, &c->own_ngrp,
-                    &c->own_lg, &c->own_sidx, &c->own_cnt, &c->Bk64, &c->Bk32, &c->tc_bk_tf32.He,
+                    &c->Bk64, &c->Bk32, &c->tc_bk_tf32.He,
                     &c->tc_bk_bf16.He, &c->ws_cx, &c->ws_cy,
-                    &c->nltc.eoff, &c->ownPx2, &c->wVs,
-                    &c->scr_main.partial, &c->scr_main.pp, &c->scr_main.W2, &c->scr_main.Wx2,
-                    &c->scr_side.partial, &c->scr_side.pp, &c->scr_side.W2, &c->scr_side.Wx2,
+                    &c->nltc.eoff, &c->wVs,
+                    &c->scr_main.partial, &c->scr_main.pp, &c->scr_main.W2,
+                    &c->scr_side.partial, &c->scr_side.pp, &c->scr_side.W2,
                     &c->ws_Y0p[0], &c->ws_Y0p[1], &c->ws_cxp[0], &c->ws_cxp[1], &c->ws_cyp[0], &c->ws_cyp[1], &c->ws_lamp[0], &c->ws_lamp[1], &c->ws_cfp[0], &c->ws_cfp[1]};
   for (DevBuf *b : bufs) b->release(&c->dev_bytes);
   for (cudaEvent_t e : c->prof.pool) cudaEventDestroy(e);

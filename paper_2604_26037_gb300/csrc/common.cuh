@@ -16,10 +16,6 @@ namespace pawfe {
 // Atoms whose projectors reach the owned nodes of one cell: the owner-cell
 // kernels stage the atom list of a cell in shared memory (checked at set-up).
 constexpr int PAIRS_PER_CELL_MAX = 192;
-// Projectors per group of the FP64 / pair-of-FP32 owner-cell nonlocal kernels: a
-// node's projectors (stored by decreasing width) are multiplied group by group up
-// to the last group with a nonzero value on the node (own_lg, own_cnt).
-constexpr int OWN_GROUP = 2;
 
 // ---------------------------------------------------------------- errors
 struct Error {
@@ -109,7 +105,7 @@ struct NlTcMats {
 // coefficients).  A context has two sets: step 2 of the next block, issued on
 // a side stream while the current block's loop runs, uses the second.
 struct NlScratch {
-  DevBuf partial, pp, W2, Wx2;
+  DevBuf partial, pp, W2;
 };
 
 // Pinned host slots for the scalar images of paw_cheb_filter's blocks.  A
@@ -204,16 +200,11 @@ struct paw_context {
   int max_own_pairs = 0;                      // largest pair count of one cell
   pawfe::DevBuf own_off;                      // int32 ncells+1
   pawfe::DevBuf own_atom;                     // int32 nown_pairs
-  pawfe::DevBuf ownP64, ownP32;               // nown_pairs * own * npad
-  pawfe::DevBuf ownPx2;                       // the same as pairs of FP32 numbers (built on first use)
+  pawfe::DevBuf ownP32;                       // nown_pairs * own * npad
   pawfe::DevBuf own_ngrp;                     // int32 per pair: projector groups of 4 with a nonzero value
-  // per pair and owned node o: index of the last projector group of 4 with a
-  // nonzero value at o (-1: none); the owned nodes sorted by that index
-  // (descending) and, per group g, the number of nodes whose index is >= g.
-  // The FP64 kernels multiply only groups that can be nonzero on a node.
-  pawfe::DevBuf own_lg;                       // int8  nown_pairs * own
-  pawfe::DevBuf own_sidx;                     // int16 nown_pairs * own
-  pawfe::DevBuf own_cnt;                      // int32 nown_pairs * npad/OWN_GROUP
+  // FP64 contractions (nonlocal_fx.cu): digit images of P for the projection and the
+  // expansion, exponent per pair and projector, node tiles with nonzero values per pair
+  pawfe::DevBuf own_proj_dg, own_exp_dg, own_sP, own_mask;
   int64_t proj_nnz = 0;                       // nonzero (owned node, projector) entries over all pairs
   pawfe::DevBuf apair_off, apair;             // atom-major list of the pairs (int32)
   // atom-pair Gram blocks G_ab = P^a^T M_D^-1 P^b for atoms with common support
@@ -323,13 +314,15 @@ void nltc_prepare(paw_context *c, cudaStream_t s);
 // the one-CTA-per-tile form writes per-pair partials PP[k][al][v] (returns false)
 bool nltc_project(paw_context *c, const float *X, int ldx, int ncols, const float *rowscale, float *PP,
                   float *U, cudaStream_t s);
-// nonlocal part of step 2 in pair-of-FP32 arithmetic (k = 0):
-// Y += sum_a P^a (C^a + cs_j C2^a) P^a^T x_j (C2, cs may be NULL), X and Y FP64
-void nl_residual_pair(paw_context *c, const double *X, int ldx, int ncols, const double *C, const double *C2,
-                      const double *cs, double *Y, int ldy, cudaStream_t s);
 // expansion with the output stage of mode (EXP_ADD / EXP_SINV / EXP_RECURRENCE)
 struct ExpArgs;
 void nltc_expand(paw_context *c, int mode, const ExpArgs &A, const float *W1, const float *W2, cudaStream_t s);
+// FP64 data (nonlocal_fx.cu): per-pair partials U[k][al][v] of P^T (rowscale .* X), and the
+// expansion; nlfx_build: the images of the pairs' P (device, nown_pairs x own x npad) at set-up
+void nlfx_build(paw_context *c, const double *P);
+void nlfx_project(paw_context *c, const double *X, int ldx, int ncols, const double *rowscale, double *U,
+                  cudaStream_t s);
+void nlfx_expand(paw_context *c, int mode, const ExpArgs &A, const double *W1, const double *W2, cudaStream_t s);
 // sum-factorised local operator on FP64 data (sumfac.cu):
 // Y += alpha * (cK K^e + cV V^e + (cM + cMcol[j]) M^e) X, cell by cell with assembly;
 void local_sf(paw_context *c, const double *X, int ldx, double *Y, int ldy, int ncols, double alpha,
@@ -360,8 +353,6 @@ void op_S(paw_context *c, const T *X, int ldx, T *Y, int ldy, int ncols,
 template <typename T>
 void op_Sinv(paw_context *c, paw_precision prec, const T *X, int ldx, T *Y, int ldy, int ncols,
              cudaStream_t s);
-// H X (which = 0) or S X (which = 1) in pair-of-FP32 arithmetic, FP64 data, k = 0
-void op_pair(paw_context *c, int which, const double *X, int ldx, double *Y, int ldy, int ncols, cudaStream_t s);
 
 // tensor-core cell products (cell_tc.cu)
 void tc_prepare(paw_context *c, paw_precision prec, cudaStream_t s);

@@ -83,18 +83,38 @@ static __device__ __noinline__ double fx_to_any(long long Y, int e) {
   return Y < 0 ? -r : r;
 }
 
-// Y 2^e as a double, rounded to nearest (ties away from zero)
-__device__ __forceinline__ double fx_to(long long Y, int e) {
-  const unsigned long long a = (unsigned long long)(Y < 0 ? -Y : Y);
-  const unsigned ah = (unsigned)(a >> 32), al = (unsigned)a;
-  const int n = __clz((int)ah);
-  const int f = 1023 + 62 - n + e;                          // exponent field less one
-  if (ah == 0 || (unsigned)f >= 2045u) return fx_to_any(Y, e);
+// (ah 2^32 + al) 2^e with the sign bit of hi, ah != 0, f = the exponent field less one in 0 .. 2044
+__device__ __forceinline__ double fx_pack(unsigned ah, unsigned al, int n, int f, unsigned hi) {
   const unsigned mh = __funnelshift_l(al, ah, n), ml = al << n;   // bit 63 set
   // 53 bits and the rounding bit; a carry moves into the exponent
   const unsigned long long q = ((unsigned long long)(mh >> 11) << 32 | __funnelshift_r(ml, mh, 11)) + ((ml >> 10) & 1u);
-  const unsigned s = ((unsigned)(Y >> 32) & 0x80000000u) + ((unsigned)f << 20);
+  const unsigned s = (hi & 0x80000000u) + ((unsigned)f << 20);
   return __longlong_as_double((long long)(q + ((unsigned long long)s << 32)));
+}
+
+// Y 2^e as a double, rounded to nearest (ties away from zero); fast for |Y| >= 2^32
+__device__ __forceinline__ double fx_to(long long Y, int e) {
+  const unsigned long long a = (unsigned long long)(Y < 0 ? -Y : Y);
+  const unsigned ah = (unsigned)(a >> 32), al = (unsigned)a;
+  const int n = __clz((int)ah), f = 1023 + 62 - n + e;
+  if (ah == 0 || (unsigned)f >= 2045u) return fx_to_any(Y, e);
+  return fx_pack(ah, al, n, f, (unsigned)(Y >> 32));
+}
+
+// the same, fast for small Y too
+__device__ __forceinline__ double fx_to_small(long long Y, int e0) {
+  int e = e0;
+  const unsigned long long a = (unsigned long long)(Y < 0 ? -Y : Y);
+  unsigned ah = (unsigned)(a >> 32), al = (unsigned)a;
+  if (ah == 0) {
+    ah = al;
+    al = 0;
+    e -= 32;
+  }
+  const int n = __clz((int)ah), f = 1023 + 62 - n + e;
+  if (ah == 0) return 0.0;
+  if ((unsigned)f >= 2045u) return fx_to_any(Y, e0);
+  return fx_pack(ah, al, n, f, (unsigned)(Y >> 32));
 }
 
 // limbs: X = fx_hi 2^32 + fx_lo with a signed low limb

@@ -1,4 +1,5 @@
-"""GPU parity of the fixed-point local operator (csrc/sumfac.cu) where its scales and tiles change.
+"""GPU parity of the fixed-point FP64 operators (csrc/sumfac.cu, csrc/nonlocal_fx.cu) where their
+scales and tiles change.
 
 Tolerance: one application is seven one-dimensional contractions; each result is exact to about
 two units of 2^-59 of the largest magnitude that the scales allow for (dropped low products and
@@ -114,3 +115,30 @@ def test_non_finite_vector_entries_reach_their_cells_only():
     assert np.isfinite(Y[:, [0, 2, 3, 5]]).all() and np.isfinite(ref).all()
     fe.close()
     fe0.close()
+
+
+@pytest.mark.parametrize("p,natoms", [(3, 2), (6, 9), (7, 9), (8, 2)])
+@pytest.mark.parametrize("ncols", [1, 16, 17, 35])
+def test_digit_contractions(p, natoms, ncols):
+    """The FP64 projector contractions on their own (the approximate inverse overlap and two steps of
+    the FP64 recurrence): tiles of 16 and 32 vectors with tails, node counts that 16 does not
+    divide, one batch of coefficients and two (nine atoms reach every cell of the small box), and
+    vectors and coefficients of very different sizes.  Operands keep 55 bits of their column's
+    largest entry, so an output is exact to a few 2^-53 of its largest entry."""
+    from oracle import cheb
+    from oracle import ops as O
+    import paper_2604_26037_gb300 as P
+    rng = np.random.default_rng(70 + p)
+    pos = rng.uniform(0.0, 5.0, (natoms, 3))
+    s = mini_system(L=5.0, n=2, p=p, positions=pos, shells=[(0, 0.4), (1, 0.35)], vdepth=1.0,
+                    D=sym_random(rng, natoms, 4, 0.1), dS=sym_random(rng, natoms, 4, 0.005))
+    op, fe = O.PawOperators(s), P.PawFE.from_system(s, block=max(ncols, 4))
+    X = rng.standard_normal((op.mesh.ndof, ncols)) * np.exp(rng.uniform(-60.0, 60.0, ncols))
+    Y, ref = fe.apply_Sinv_approx(to_dev(X)).cpu().numpy(), op.apply_Sinv_approx(X)
+    F = fe.cheb_filter(to_dev(X), np.linspace(0.1, 0.9, ncols), 3, (0.0, 1.0, 400.0), prec="fp64").cpu().numpy()
+    Fr = cheb.rchfsi_filter(op.apply_H, op.apply_S, op.apply_Sinv_approx, X, np.linspace(0.1, 0.9, ncols), 3, 0.0, 1.0,
+                            400.0)
+    for j in range(ncols):
+        assert rel_err(Y[:, j], ref[:, j]) < TOL
+        assert rel_err(F[:, j], Fr[:, j]) < TOL
+    fe.close()
