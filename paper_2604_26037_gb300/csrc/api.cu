@@ -788,48 +788,38 @@ __global__ void k_random_vec(int64_t n, uint64_t seed, double *__restrict__ v) {
 }
 
 // ============================================================== gradient kernels
-// dV[e][q] = wq[q] * sum_v f[v] (sum_I Nq[q][I] X[dof_e(I)][v])^2, one block per cell
-// (wq NULL: 1, the values at the points; f NULL: 1)
-template <typename T>
-__global__ void __launch_bounds__(256) k_grad_V(int nc, int nq, const int *__restrict__ cell_dofs,
-                                                const double *__restrict__ Nq, const double *__restrict__ wq,
-                                                const T *__restrict__ X, int ldx, int ncols,
-                                                const double *__restrict__ f, double *__restrict__ dV) {
-  extern __shared__ double xs[];   // [nc][32]
-  const int e = blockIdx.x;
-  const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
-  for (int q = threadIdx.x; q < nq; q += blockDim.x) dV[(size_t)e * nq + q] = 0.0;
-  for (int v0 = 0; v0 < ncols; v0 += 32) {
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < nc * 32; idx += blockDim.x) {
-      const int I = idx >> 5, v = idx & 31;
-      xs[idx] = (v0 + v < ncols) ? (double)X[(size_t)cell_dofs[(size_t)e * nc + I] * ldx + v0 + v] : 0.0;
-    }
-    __syncthreads();
-    const double fv = (f && v0 + lane < ncols) ? f[v0 + lane] : 1.0;
-    for (int q = grp; q < nq; q += 8) {
-      double u = 0.0;
-      for (int I = 0; I < nc; ++I) u += Nq[(size_t)q * nc + I] * xs[I * 32 + lane];
-      double s = fv * u * u;
-      for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-      if (lane == 0) dV[(size_t)e * nq + q] += (wq ? wq[q] : 1.0) * s;
-    }
-  }
-}
-
 // dD[a][ext(al)][ext(be)] = sum_v f[v] U[a][al][v] U[a][be][v]  (ext: internal -> caller's
 // projector index; f NULL: 1)
 template <typename T>
-__global__ void k_grad_D(int npj, int npad, const T *__restrict__ U, int ldu, int ncols, const int *__restrict__ ext,
-                         const double *__restrict__ f, double *__restrict__ dD) {
-  const int a = blockIdx.x;
-  for (int o = threadIdx.x; o < npj * npj; o += blockDim.x) {
-    const int al = o / npj, be = o % npj;
-    double s = 0.0;
-    for (int v = 0; v < ncols; ++v)
-      s += (f ? f[v] : 1.0) * (double)U[((size_t)a * npad + al) * ldu + v] *
-           (double)U[((size_t)a * npad + be) * ldu + v];
-    dD[(size_t)a * npj * npj + (size_t)ext[al] * npj + ext[be]] = s;
+__global__ void __launch_bounds__(256) k_grad_D(int npj, int npad, const T *__restrict__ U, int ldu, int ncols,
+                                                const int *__restrict__ ext, const double *__restrict__ f,
+                                                double *__restrict__ dD) {
+  constexpr int VC = 32;                // vectors staged at a time, the rows one entry apart in banks
+  __shared__ double su[32 * (VC + 1)], sf[VC];
+  const int a = blockIdx.x, nout = npj * npj;
+  constexpr int PER = 4;                // up to 32 x 32 outputs over 256 threads
+  double s[PER] = {0.0, 0.0, 0.0, 0.0};
+  for (int v0 = 0; v0 < ncols; v0 += VC) {
+    const int nv = min(VC, ncols - v0);
+    if (v0) __syncthreads();
+    for (int i = threadIdx.x; i < npj * VC; i += 256) {
+      const int al = i / VC, v = i % VC;
+      su[al * (VC + 1) + v] = v < nv ? (double)U[((size_t)a * npad + al) * ldu + v0 + v] : 0.0;
+    }
+    if (threadIdx.x < VC) sf[threadIdx.x] = (f && threadIdx.x < nv) ? f[v0 + threadIdx.x] : 1.0;
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+      const int o = threadIdx.x + j * 256;
+      if (o >= nout) break;
+      const double *x = su + (o / npj) * (VC + 1), *y = su + (o % npj) * (VC + 1);
+      for (int v = 0; v < nv; ++v) s[j] += (f ? sf[v] * x[v] : x[v]) * y[v];
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < PER; ++j) {
+    const int o = threadIdx.x + j * 256;
+    if (o < nout) dD[(size_t)a * nout + (size_t)ext[o / npj] * npj + ext[o % npj]] = s[j];
   }
 }
 
@@ -1464,17 +1454,10 @@ paw_status paw_energy(paw_handle c, paw_precision prec, const void *X, int ld, i
 // outV[e][q] = wq[q] sum_v f[v] u_v(x_q)^2 and outD[a] = sum_v f[v] U_v U_v^T (wq, f optional)
 static void density_like(paw_context *c, paw_precision prec, const void *X, int ld, int N, const double *wq,
                          const double *f, double *outV, double *outD, cudaStream_t s) {
-  const size_t shm = sizeof(double) * c->nc * 32;
-  if (prec == PAW_FP64) {
-    PAW_CUDA(cudaFuncSetAttribute(k_grad_V<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
-    k_grad_V<double><<<c->ncells, 256, shm, s>>>(c->nc, c->nq, c->cell_dofs.as<int>(), c->Nq64.as<double>(), wq,
-                                                  (const double *)X, ld, N, f, outV);
-  } else {
-    PAW_CUDA(cudaFuncSetAttribute(k_grad_V<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
-    k_grad_V<float><<<c->ncells, 256, shm, s>>>(c->nc, c->nq, c->cell_dofs.as<int>(), c->Nq64.as<double>(), wq,
-                                                 (const float *)X, ld, N, f, outV);
-  }
-  PAW_LAUNCH_CHECK("k_grad_V");
+  if (prec == PAW_FP64)
+    density_sf<double>(c, (const double *)X, ld, N, wq, f, outV, s);
+  else
+    density_sf<float>(c, (const float *)X, ld, N, wq, f, outV, s);
   if (c->nown_pairs > 0 && outD) {
     if (prec == PAW_FP64) {
       c->scr->W2.ensure(sizeof(double) * (size_t)c->natoms * c->npad * N, &c->dev_bytes);

@@ -327,6 +327,10 @@ void nlfx_expand(paw_context *c, int mode, const ExpArgs &A, const double *W1, c
 // Y += alpha * (cK K^e + cV V^e + (cM + cMcol[j]) M^e) X, cell by cell with assembly;
 void local_sf(paw_context *c, const double *X, int ldx, double *Y, int ldy, int ncols, double alpha,
               double cK, double cV, double cM, const double *cMcol, cudaStream_t s);
+// out[e][q] = wq[q] sum_v f[v] u_v(x_q)^2 at the (p+2)^3 Gauss points of every cell (wq, f NULL: 1)
+template <typename T>
+void density_sf(paw_context *c, const T *X, int ldx, int ncols, const double *wq, const double *f, double *out,
+                cudaStream_t s);
 // FP64 sum-factorised Bloch term: Y += alpha * B X, B = sum_d k_d G_d cell by cell
 // (G_d the skew cell form of int N_I dN_J/dx_d, Eq. hij), with assembly
 void bloch_sf(paw_context *c, const double *X, int ldx, double *Y, int ldy, int ncols, double alpha,

@@ -74,6 +74,20 @@ __device__ __forceinline__ long long fx_from(double x, int E) {
   return (int)hi < 0 ? -t : t;
 }
 
+// the same for FP32 numbers (fields of the equal FP64 numbers)
+__device__ __forceinline__ int fx_field(float x) {
+  const int f = (int)(__float_as_uint(x) >> 23) & 0xff;
+  return f == 0xff ? 0x7ff : max(f, 1) + 896;
+}
+template <int BITS = FX_F>
+__device__ __forceinline__ long long fx_from(float x, int E) {
+  const unsigned b = __float_as_uint(x);
+  const int f = (int)(b >> 23) & 0xff;
+  const unsigned long long m = (unsigned long long)((b & 0x7fffffu) | (f ? 0x800000u : 0u)) << (BITS - 24);
+  const long long t = (long long)(m >> min(E - (max(f, 1) + 896), 63));
+  return (int)b < 0 ? -t : t;
+}
+
 // Y 2^e as a double (any Y and e)
 static __device__ __noinline__ double fx_to_any(long long Y, int e) {
   if (Y == 0) return 0.0;

@@ -142,3 +142,21 @@ def test_digit_contractions(p, natoms, ncols):
         assert rel_err(Y[:, j], ref[:, j]) < TOL
         assert rel_err(F[:, j], Fr[:, j]) < TOL
     fe.close()
+
+
+@pytest.mark.parametrize("p", [1, 2, 4, 6, 7, 8])
+@pytest.mark.parametrize("ncols,prec", [(1, "fp64"), (9, "fp64"), (4, "fp32"), (33, "fp32")])
+def test_density(p, ncols, prec):
+    """Densities and occupation matrices with occupations of both signs; FP32 vectors enter exactly,
+    their projector coefficients are FP32 sums (1e-5)."""
+    import torch
+    from oracle import grad
+    op, fe = _oracle(p), _fe(p)
+    rng = np.random.default_rng(10 * p + ncols)
+    X, f = rng.standard_normal((op.mesh.ndof, ncols)), rng.uniform(-1.0, 2.0, ncols)
+    Xd = to_dev(X, torch.float64 if prec == "fp64" else torch.float32)
+    rho, D = grad.density(op, Xd.double().cpu().numpy(), f)
+    r, d = fe.density(Xd, occ=f, prec=prec)
+    assert rel_err(r.cpu().numpy(), rho) < TOL
+    assert rel_err(d.cpu().numpy(), D) < (TOL if prec == "fp64" else 1e-5)
+    fe.close()
