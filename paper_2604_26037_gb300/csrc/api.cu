@@ -262,8 +262,8 @@ static void merge_cplx(paw_context *c, const T *Xs, int n, T *Z, int ldz, cudaSt
 
 // Y = H X - S X Lambda in FP64 (Algorithm 2 step 2)
 static void residual_block(paw_context *c, const double *X, int ldx, const double *negLam_dev,
-                           double *Y, int ldy, int ncols, cudaStream_t s) {
-  zero_block<double>(Y, c->ndof, ncols, ldy, s);
+                           double *Y, int ldy, int ncols, cudaStream_t s, int nzero = 0) {
+  zero_block<double>(Y, c->ndof, std::max(ncols, nzero), ldy, s);   // (columns past ncols stay zero)
   // both parts add into Y (the local part first: with the nonlocal part first beside a
   // loop, the mid filter call measured 293 instead of 288 ms)
   auto nonlocal = [&]() {
@@ -366,7 +366,25 @@ __global__ void k_stage_scalars(const double *__restrict__ hd, double *__restric
   }
 }
 
-static void block_step2(paw_context *c, const double *X, int ldx, int nb, const ChebScalars &S, const double *hd,
+// Columns that the loop works on for a block of nb: the persistent tensor-core kernels copy whole
+// 16-byte rows, so a block of FP32 R that four does not divide is filtered with up to three zero
+// columns beside it (degree 6, 12^3 cells, 45 columns, 20 steps: 13.9 ms, 28.9 ms with the
+// one-CTA-per-tile kernels and the earlier step 2; 10^3 cells of degree 5, 301 columns in blocks
+// of 128, BF16: 16.4 and 20.2 ms).  Not at k != 0, whose two halves would each need padding, and
+// not where the tiles of a cell product fit the SMs twice over: there the one-CTA-per-tile
+// kernels add the cells in nearly the same order on every call, and so they stay.
+static int cheb_cols(const paw_context *c, paw_precision prec, int nb) {
+  const bool tc = prec == PAW_TF32 || prec == PAW_BF16;
+  const int64_t tiles = (int64_t)c->ncells * ((nb + 127) / 128);
+  return (tc && !c->kc && c->tc_variant == 0 && tiles > 304) ? (nb + 3) / 4 * 4 : nb;
+}
+struct PaddedIssue {
+  paw_context *c;
+  PaddedIssue(paw_context *ctx, int mode) : c(ctx) { c->padded = mode; }
+  ~PaddedIssue() { c->padded = PAD_NONE; }
+};
+
+static void block_step2(paw_context *c, const double *X, int ldx, int nb, int nbp, const ChebScalars &S, const double *hd,
                         const float *hf, int par, cudaStream_t s, const double *hd_dev, const float *hf_dev) {
   c->ws_lamp[par].ensure(sizeof(double) * S.nd, &c->dev_bytes);
   c->ws_cfp[par].ensure(sizeof(float) * S.nf, &c->dev_bytes);
@@ -380,14 +398,15 @@ static void block_step2(paw_context *c, const double *X, int ldx, int nb, const 
     PAW_CUDA(cudaMemcpyAsync(c->ws_lamp[par].ptr, hd, sizeof(double) * S.nd, cudaMemcpyHostToDevice, s));
     PAW_CUDA(cudaMemcpyAsync(c->ws_cfp[par].ptr, hf, sizeof(float) * S.nf, cudaMemcpyHostToDevice, s));
   }
-  c->ws_Y0p[par].ensure(sizeof(double) * c->ndof * nb, &c->dev_bytes);
+  c->ws_Y0p[par].ensure(sizeof(double) * c->ndof * nbp, &c->dev_bytes);
   // step 2: Y = H X - S X Lambda (FP64; phases 0 and 4)
-  residual_block(c, X, ldx, c->ws_lamp[par].as<double>(), c->ws_Y0p[par].as<double>(), nb, nb, s);
+  residual_block(c, X, ldx, c->ws_lamp[par].as<double>(), c->ws_Y0p[par].as<double>(), nbp, nb, s, nbp);
 }
 
 template <typename TR>
-static void block_loop(paw_context *c, paw_precision prec, const double *X, int ldx, int nb, double a0, double cc,
-                       const ChebScalars &S, int par, double *Xo, int ldo, cudaStream_t s) {
+static void block_loop(paw_context *c, paw_precision prec, const double *X, int ldx, int nout, int nb, double a0,
+                       double cc, const ChebScalars &S, int par, double *Xo, int ldo, cudaStream_t s) {
+  const PaddedIssue padded(c, nb != nout ? PAD_SAME : PAD_NONE);   // nb columns are worked on, nout belong to the block
   const int64_t M = c->ndof;
   const int nsteps = S.nsteps;
   const double *d_neglam = c->ws_lamp[par].as<double>();
@@ -471,20 +490,20 @@ static void block_loop(paw_context *c, paw_precision prec, const double *X, int 
   {
     PhaseScope ps(c, 5, s);
     op_Sinv<TR>(c, prec, RY, ldr, T, ldr, nb, s);
-    k_cheb_recover<TR><<<ew_grid(M, nb), blk, 0, s>>>(M, nb, T, ldr, X, ldx, d_lyfin, Xo, ldo);
+    k_cheb_recover<TR><<<ew_grid(M, nout), blk, 0, s>>>(M, nout, T, ldr, X, ldx, d_lyfin, Xo, ldo);
     PAW_LAUNCH_CHECK("k_cheb_recover");
   }
 }
 
-void cheb_issue(paw_context *c, paw_precision prec, const double *X, int ldx, int nb, paw_bounds bd,
+void cheb_issue(paw_context *c, paw_precision prec, const double *X, int ldx, int nb, int nbp, paw_bounds bd,
                 const ChebScalars &S, const double *hd, const float *hf, double *Xo, int ldo, cudaStream_t s,
                 const double *hd_dev, const float *hf_dev) {
   const double cc = (bd.bU + bd.bW) / 2.0;
-  block_step2(c, X, ldx, nb, S, hd, hf, 0, s, hd_dev, hf_dev);
+  block_step2(c, X, ldx, nb, nbp, S, hd, hf, 0, s, hd_dev, hf_dev);
   if (prec == PAW_FP64)
-    block_loop<double>(c, prec, X, ldx, nb, bd.a0, cc, S, 0, Xo, ldo, s);
+    block_loop<double>(c, prec, X, ldx, nb, nbp, bd.a0, cc, S, 0, Xo, ldo, s);
   else
-    block_loop<float>(c, prec, X, ldx, nb, bd.a0, cc, S, 0, Xo, ldo, s);
+    block_loop<float>(c, prec, X, ldx, nb, nbp, bd.a0, cc, S, 0, Xo, ldo, s);
 }
 
 // Next slot of the handle's pinned ring, large enough for `bytes`.  Waits only
@@ -527,14 +546,17 @@ static void release_ring(paw_context *c) {
 static void cheb_block(paw_context *c, paw_precision prec, const double *X, int ldx, const double *lam, int nb,
                        int m, paw_bounds bd, double *Xo, int ldo, cudaStream_t s) {
   ChebScalars S;
-  const size_t nd = cheb_nd(nb, m), nf = cheb_nf(nb, m);
+  const int nbp = cheb_cols(c, prec, nb);
+  const size_t nd = cheb_nd(nbp, m), nf = cheb_nf(nbp, m);
   HostSlot &sl = acquire_slot(c, sizeof(double) * nd + sizeof(float) * nf);
   double *hd = static_cast<double *>(sl.host);
   float *hf = reinterpret_cast<float *>(hd + nd);
-  cheb_plan(nb, m, bd, lam, S, hd, hf);
+  std::vector<double> lamp(lam, lam + nb);
+  lamp.resize(nbp, lam[nb - 1]);
+  cheb_plan(nbp, m, bd, lamp.data(), S, hd, hf);
   const double *hd_dev = static_cast<const double *>(sl.dev);
   try {
-    cheb_issue(c, prec, X, ldx, nb, bd, S, hd, hf, Xo, ldo, s, hd_dev, reinterpret_cast<const float *>(hd_dev + nd));
+    cheb_issue(c, prec, X, ldx, nb, nbp, bd, S, hd, hf, Xo, ldo, s, hd_dev, reinterpret_cast<const float *>(hd_dev + nd));
   } catch (...) {
     // copies from the slot may already be enqueued: keep it until the stream passes them
     if (cudaEventRecord(sl.done, s) == cudaSuccess) sl.pending = true;
@@ -545,17 +567,15 @@ static void cheb_block(paw_context *c, paw_precision prec, const double *X, int 
 }
 
 // ============================================================== overlapped blocks
-// Step 2 (FP64, bound by the FP64 pipe) of block j + 1 runs on a low-priority
-// side stream while the loop of block j (bound by copy bandwidth and the
-// tensor cores) runs on a high-priority stream: the blocks are independent
-// (Sec. 4.4 filters blocks independently), so this reorders nothing but the
-// schedule.  While a step 2 shares the SMs, the loop's persistent
-// cell-product and projection kernels take their half-shared-memory form and
-// the FP64 local kernel its 4-vector form, so that one CTA of each fits on
-// an SM; the high priority hands freed SM slots to the persistent kernels
-// first.  Blocks of parity j & 1 use the parity's Y buffer and scalar
-// images; the side stream reuses them for block j + 2 only after the loop of
-// block j has finished.
+// Step 2 of block j + 1 runs on a low-priority side stream while the loop of block j runs on a
+// high-priority stream: the blocks are independent (Sec. 4.4 filters blocks independently), so
+// this reorders nothing but the schedule.  The kernels of the loop fill the shared memory of
+// their SMs, so step 2 advances where they leave SMs idle (at their ends and in small problems):
+// 1-7% per call.  (Forms of the loop kernels with half the shared memory, beside which blocks of
+// step 2 fit, were 24% slower and hid an FP64-pipe-bound step 2 of 78 ms per 256 vectors; beside
+// the present one of 18 ms the mid call takes 190.5 ms with them and 186.1 ms without.)  Blocks
+// of parity j & 1 use the parity's Y buffer and scalar images; the side stream reuses them for
+// block j + 2 only after the loop of block j has finished.
 static cudaEvent_t next_event(paw_context *c) {
   if (c->ev_used == c->ev_pool.size()) {
     cudaEvent_t e;
@@ -573,23 +593,11 @@ static void ensure_streams(paw_context *c) {
   PAW_CUDA(cudaStreamCreateWithPriority(&c->s_side, cudaStreamNonBlocking, least));
 }
 
-// work issued while this is alive uses the side scratch set and the lean FP64 kernel
+// work issued while this is alive uses the side scratch set
 struct SideIssue {
   paw_context *c;
-  SideIssue(paw_context *ctx, bool lean) : c(ctx) {
-    c->scr = &c->scr_side;
-    c->sf_lean = lean ? 1 : 0;
-  }
-  ~SideIssue() {
-    c->scr = &c->scr_main;
-    c->sf_lean = 0;
-  }
-};
-
-struct LeanLoop {
-  paw_context *c;
-  LeanLoop(paw_context *ctx, bool lean) : c(ctx) { c->lean = lean ? 1 : 0; }
-  ~LeanLoop() { c->lean = 0; }
+  explicit SideIssue(paw_context *ctx) : c(ctx) { c->scr = &c->scr_side; }
+  ~SideIssue() { c->scr = &c->scr_main; }
 };
 
 static void cheb_filter_overlapped(paw_context *c, paw_precision prec, const double *X, int ldx, const double *lam,
@@ -617,24 +625,20 @@ static void cheb_filter_overlapped(paw_context *c, paw_precision prec, const dou
     return c->kc ? c->ws_cxp[j & 1].as<double>() : X + (size_t)j * B;
   };
   auto issue_step2 = [&](int j) {
-    const int j0 = j * B, nb = std::min(B, ncols - j0), nr = cw * nb;
-    const size_t nd = cheb_nd(nr, m), nf = cheb_nf(nr, m);
+    const int j0 = j * B, nb = std::min(B, ncols - j0), nr = cw * nb, nrp = cheb_cols(c, prec, nr);
+    const size_t nd = cheb_nd(nrp, m), nf = cheb_nf(nrp, m);
     HostSlot &sl = acquire_slot(c, sizeof(double) * nd + sizeof(float) * nf);
     double *hd = static_cast<double *>(sl.host);
     float *hf = reinterpret_cast<float *>(hd + nd);
-    if (c->kc) {
-      std::vector<double> lam2(2 * (size_t)nb);
-      for (int i = 0; i < nb; ++i) lam2[i] = lam2[nb + i] = lam[j0 + i];
-      cheb_plan(nr, m, bd, lam2.data(), S[j], hd, hf);
-    } else {
-      cheb_plan(nr, m, bd, lam + j0, S[j], hd, hf);
-    }
+    std::vector<double> lamr(nrp, lam[j0 + nb - 1]);
+    for (int i = 0; i < nr; ++i) lamr[i] = lam[j0 + i % nb];
+    cheb_plan(nrp, m, bd, lamr.data(), S[j], hd, hf);
     if (j >= 2) PAW_CUDA(cudaStreamWaitEvent(c->s_side, evFree[j - 2], 0));   // parity buffers free again
     try {
-      SideIssue side(c, j > 0);
+      const SideIssue side(c);
       const double *hd_dev = static_cast<const double *>(sl.dev);
       if (c->kc) split_cplx<double>(c, X + 2 * (size_t)j0, ldx, nb, c->ws_cxp[j & 1].as<double>(), c->s_side);
-      block_step2(c, block_in(j), c->kc ? nr : ldx, nr, S[j], hd, hf, j & 1, c->s_side, hd_dev,
+      block_step2(c, block_in(j), c->kc ? nr : ldx, nr, nrp, S[j], hd, hf, j & 1, c->s_side, hd_dev,
                   reinterpret_cast<const float *>(hd_dev + nd));
     } catch (...) {
       if (cudaEventRecord(sl.done, c->s_side) == cudaSuccess) sl.pending = true;
@@ -650,15 +654,13 @@ static void cheb_filter_overlapped(paw_context *c, paw_precision prec, const dou
     if (j + 1 < nbk) issue_step2(j + 1);
     const int j0 = j * B, nb = std::min(B, ncols - j0), nr = cw * nb;
     PAW_CUDA(cudaStreamWaitEvent(c->s_loop, evY[j], 0));
-    {
-      LeanLoop lean(c, j + 1 < nbk);   // a step 2 shares the SMs with this loop
-      if (c->kc) {
-        double *Y = c->ws_cyp[j & 1].as<double>();
-        block_loop<float>(c, prec, block_in(j), nr, nr, bd.a0, cc, S[j], j & 1, Y, nr, c->s_loop);
-        merge_cplx<double>(c, Y, nb, Xo + 2 * (size_t)j0, ldo, c->s_loop);
-      } else {
-        block_loop<float>(c, prec, X + j0, ldx, nb, bd.a0, cc, S[j], j & 1, Xo + j0, ldo, c->s_loop);
-      }
+    if (c->kc) {
+      double *Y = c->ws_cyp[j & 1].as<double>();
+      block_loop<float>(c, prec, block_in(j), nr, nr, nr, bd.a0, cc, S[j], j & 1, Y, nr, c->s_loop);
+      merge_cplx<double>(c, Y, nb, Xo + 2 * (size_t)j0, ldo, c->s_loop);
+    } else {
+      block_loop<float>(c, prec, X + j0, ldx, nb, cheb_cols(c, prec, nb), bd.a0, cc, S[j], j & 1, Xo + j0, ldo,
+                        c->s_loop);
     }
     evFree[j] = next_event(c);
     PAW_CUDA(cudaEventRecord(evFree[j], c->s_loop));
@@ -886,6 +888,18 @@ static void apply_cplx(paw_context *c, paw_precision prec, int which, const T *X
   merge_cplx<T>(c, ys, ncols, Y, ldy, s);
 }
 
+// dst[i][v] = src[i][v] for v < n, 0 for n <= v < m
+__global__ void k_copy_rows(int64_t rows, const float *__restrict__ src, int lds, int n, float *__restrict__ dst,
+                            int ldd, int m) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.y + threadIdx.y;
+  if (i >= rows) return;
+  for (int v = threadIdx.x; v < m; v += blockDim.x) dst[i * ldd + v] = v < n ? src[i * lds + v] : 0.f;
+}
+static void copy_rows(const float *src, int lds, int n, float *dst, int ldd, int m, int64_t rows, cudaStream_t s) {
+  k_copy_rows<<<(unsigned)((rows + 7) / 8), dim3(32, 8), 0, s>>>(rows, src, lds, n, dst, ldd, m);
+  PAW_LAUNCH_CHECK("k_copy_rows");
+}
+
 static void apply_any(paw_context *c, paw_precision prec, int which, const void *X, int ldx, void *Y, int ldy,
                       int ncols, cudaStream_t s) {
   if (prec == PAW_F32X2) {
@@ -897,6 +911,25 @@ static void apply_any(paw_context *c, paw_precision prec, int which, const void 
       apply_cplx<double>(c, prec, which, (const double *)X, ldx, (double *)Y, ldy, ncols, s);
     else
       apply_cplx<float>(c, prec, which, (const float *)X, ldx, (float *)Y, ldy, ncols, s);
+    return;
+  }
+  const bool rows16 = ncols % 4 == 0 && ldx % 4 == 0 && ldy % 4 == 0 && ((uintptr_t)X | (uintptr_t)Y) % 16 == 0;
+  if ((prec == PAW_TF32 || prec == PAW_BF16) && which != 1 && !rows16 && c->nown_pairs > 0 &&
+      c->tc_variant == 0) {
+    // rows that are not whole 16-byte pieces: through zero-padded copies, on which the persistent
+    // tensor-core kernels run (approximate inverse overlap, degree 6, 12^3 cells, 130 columns: 0.67
+    // instead of 1.03 ms; H 1.14 instead of 1.69 ms; no slower on 4^3 cells of degree 4)
+    const int np = (ncols + 3) / 4 * 4;
+    c->ws_cx.ensure(sizeof(float) * (size_t)c->ndof * np, &c->dev_bytes);
+    c->ws_cy.ensure(sizeof(float) * (size_t)c->ndof * np, &c->dev_bytes);
+    float *xs = c->ws_cx.as<float>(), *ys = c->ws_cy.as<float>();
+    const PaddedIssue padded(c, PAD_CELL);
+    copy_rows((const float *)X, ldx, ncols, xs, np, np, c->ndof, s);
+    if (which == 0)
+      op_H<float>(c, prec, xs, np, ys, np, np, s);
+    else
+      op_Sinv<float>(c, prec, xs, np, ys, np, np, s);
+    copy_rows(ys, np, ncols, (float *)Y, ldy, ncols, c->ndof, s);
     return;
   }
   if (prec == PAW_FP64) {

@@ -96,7 +96,7 @@ void issue_instance(paw_batch_s *b, paw_precision prec, const paw_batch_problem 
   const int B = c->opts.block;
   for (size_t k = 0; k < P.blocks.size(); ++k) {
     const int j0 = (int)k * B, nb = std::min(B, q.ncols - j0);
-    pawfe::cheb_issue(c, prec, q.X_in + j0, q.ldx, nb, q.bounds, P.blocks[k], b->hd + P.hd_off[k],
+    pawfe::cheb_issue(c, prec, q.X_in + j0, q.ldx, nb, nb, q.bounds, P.blocks[k], b->hd + P.hd_off[k],
                       b->hf + P.hf_off[k], q.X_out + j0, q.ldo, s);
   }
 }
@@ -196,9 +196,9 @@ void tune_instance(paw_batch_s *b, paw_precision prec, const paw_batch_problem &
   int bestv = 0;
   for (int v = 0; v < 2; ++v) {
     c->tc_variant = v;
-    pawfe::cheb_issue(c, prec, q.X_in, q.ldx, nb, q.bounds, S, hd.data(), hf.data(), q.X_out, q.ldo, s);   // warm
+    pawfe::cheb_issue(c, prec, q.X_in, q.ldx, nb, nb, q.bounds, S, hd.data(), hf.data(), q.X_out, q.ldo, s);   // warm
     PAW_CUDA(cudaEventRecord(e0, s));
-    pawfe::cheb_issue(c, prec, q.X_in, q.ldx, nb, q.bounds, S, hd.data(), hf.data(), q.X_out, q.ldo, s);
+    pawfe::cheb_issue(c, prec, q.X_in, q.ldx, nb, nb, q.bounds, S, hd.data(), hf.data(), q.X_out, q.ldo, s);
     PAW_CUDA(cudaEventRecord(e1, s));
     PAW_CUDA(cudaEventSynchronize(e1));
     float ms = 0.f;

@@ -253,16 +253,17 @@ __global__ void k_tile_mats(const float *__restrict__ He, long long stride, int 
 // Persistent warp-specialised form (tc_stream.cuh) for 16-byte-aligned rows:
 // tile = (cell, 128 vectors), one accumulation round per N tile of H^e.
 // SMALL: N tiles of at most 176 rows (degree <= 6), which leaves room for one
-// more pipeline stage.  LEAN: two stages (about half the shared memory), the
-// form used while an FP64 step 2 shares the SMs (paw_cheb_filter).
-template <bool BF, bool SMALL, bool LEAN = false>
+// more pipeline stage.  TR: vectors enter as the TF32 part of their FP32 values
+// (as in k_cell_tc) instead of rounded, for blocks padded to whole 16-byte rows,
+// whose results then do not depend on the kernel family.
+template <bool BF, bool SMALL, bool TR>
 struct CellStream {
-  static constexpr int NW = 1, NEPI = 8;
-  static constexpr int S = LEAN ? 2 : (BF ? 2 : 3) + (SMALL ? 1 : 0);
-  static constexpr bool BF16 = BF;
+  static constexpr int NEPI = 8;
+  static constexpr int S = (BF ? 2 : 3) + (SMALL ? 1 : 0);
+  static constexpr bool BF16 = BF, TRUNC = TR, SCALED = false;
   static constexpr uint32_t B_MAX = (SMALL ? 176u : 256u) * 128u;
   static constexpr int KR = BF ? 64 : 32;
-  CUtensorMap tm[NW];   // rows of X (gathered with TMA)
+  CUtensorMap tm;       // rows of X (gathered with TMA)
   int ntiles, ncols, vtiles, nc, ntile, ntiles_n, kchunks, ldx, ldy;
   size_t cell_bytes;
   const uint8_t *Ht;
@@ -284,14 +285,13 @@ struct CellStream {
   __device__ int nchunks(const Tile &, int) const { return kchunks; }
   __device__ int ncol(const Tile &, int) const { return ntile; }
   __device__ int xcol(const Tile &T) const { return T.vt * MT; }
-  __device__ int row_id(const Tile &T, int, int kc, int j, int) const {
+  __device__ int row_id(const Tile &T, int, int kc, int j) const {
     const int k = kc * KR + j;
     return k < nc ? cell_dofs[(size_t)T.e * nc + k] : -1;
   }
   __device__ const uint8_t *bsrc(const Tile &T, int sub, int kc) const {
     return Ht + (size_t)T.e * cell_bytes + ((size_t)sub * kchunks + kc) * ntile * 128;
   }
-  __device__ uint32_t dcol(int) const { return 0; }
   // Y[dof(n)][v] += alpha D[v][n]: coalesced FP32 reductions, one node row per warp instruction
   __device__ void epilogue(const Tile &T, int sub, uint32_t tl, int q, int part, int lane, bool) const {
     const int ng = ntile / 16, per = (ng + 1) / 2;
@@ -360,10 +360,11 @@ size_t tc_smem_bytes(int ntile, int kchunks, bool bf16) {
   return b < 80 * 1024 ? 80 * 1024 : b;
 }
 
-template <bool BF, bool SMALL, bool LEAN>
+template <bool BF, bool SMALL, bool TR>
 static void cell_stream(paw_context *c, const TcMats &T, const float *X, int ldx, float *Y, int ldy, int ncols,
                         float alpha, cudaStream_t s) {
-  CellStream<BF, SMALL, LEAN> p;
+  using P = CellStream<BF, SMALL, TR>;
+  P p;
   p.vtiles = (ncols + MT - 1) / MT;
   const int64_t nt = (int64_t)c->ncells * p.vtiles;
   PAW_REQUIRE(nt < (1ll << 31), PAW_ERR_UNSUPPORTED, "too many cell tiles");
@@ -381,13 +382,9 @@ static void cell_stream(paw_context *c, const TcMats &T, const float *X, int ldx
   p.X = X;
   p.Y = Y;
   p.alpha = alpha;
-  encode_row_map(&p.tm[0], X, c->ndof, ncols, ldx);
-  using P = CellStream<BF, SMALL, LEAN>;
+  encode_row_map(&p.tm, X, c->ndof, ncols, ldx);
   const size_t shm = tcs::Geo<P>::SMEM;
   PAW_CUDA(cudaFuncSetAttribute(tcs::k_tc_stream<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
-  if (LEAN)   // the whole shared memory configured, so that an FP64 CTA fits beside this one
-    PAW_CUDA(cudaFuncSetAttribute(tcs::k_tc_stream<P>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                  cudaSharedmemCarveoutMaxShared));
   int dev = 0, nsm = 0;
   PAW_CUDA(cudaGetDevice(&dev));
   PAW_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
@@ -409,25 +406,15 @@ static void cell_apply_tc_mats(paw_context *c, paw_precision prec, const TcMats 
   if (c->tc_variant == 0 && reinterpret_cast<uintptr_t>(X) % 16 == 0 && ldx % 4 == 0 && ncols % 4 == 0 &&
       Tm.ntile <= 256) {
     const bool small = Tm.ntile <= 176;
-    if (c->lean) {   // an FP64 step 2 shares the SMs: half the shared memory
-      if (bf16)
-        small ? cell_stream<true, true, true>(c, Tm, X, ldx, Y, ldy, ncols, alpha, s)
-              : cell_stream<true, false, true>(c, Tm, X, ldx, Y, ldy, ncols, alpha, s);
-      else
-        small ? cell_stream<false, true, true>(c, Tm, X, ldx, Y, ldy, ncols, alpha, s)
-              : cell_stream<false, false, true>(c, Tm, X, ldx, Y, ldy, ncols, alpha, s);
-      return;
-    }
     if (bf16) {
-      if (small)
-        cell_stream<true, true, false>(c, Tm, X, ldx, Y, ldy, ncols, alpha, s);
-      else
-        cell_stream<true, false, false>(c, Tm, X, ldx, Y, ldy, ncols, alpha, s);
+      small ? cell_stream<true, true, false>(c, Tm, X, ldx, Y, ldy, ncols, alpha, s)
+            : cell_stream<true, false, false>(c, Tm, X, ldx, Y, ldy, ncols, alpha, s);
+    } else if (c->padded) {
+      small ? cell_stream<false, true, true>(c, Tm, X, ldx, Y, ldy, ncols, alpha, s)
+            : cell_stream<false, false, true>(c, Tm, X, ldx, Y, ldy, ncols, alpha, s);
     } else {
-      if (small)
-        cell_stream<false, true, false>(c, Tm, X, ldx, Y, ldy, ncols, alpha, s);
-      else
-        cell_stream<false, false, false>(c, Tm, X, ldx, Y, ldy, ncols, alpha, s);
+      small ? cell_stream<false, true, false>(c, Tm, X, ldx, Y, ldy, ncols, alpha, s)
+            : cell_stream<false, false, false>(c, Tm, X, ldx, Y, ldy, ncols, alpha, s);
     }
     return;
   }

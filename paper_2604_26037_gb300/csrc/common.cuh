@@ -17,6 +17,11 @@ namespace pawfe {
 // kernels stage the atom list of a cell in shared memory (checked at set-up).
 constexpr int PAIRS_PER_CELL_MAX = 192;
 
+// Blocks whose rows are not whole 16-byte pieces are padded for the persistent tensor-core kernels,
+// which then round the vectors as the one-CTA-per-tile kernels do: in the cell products (both), and
+// with M_D^-1 applied before the rounding of a projection (PAD_SAME, the filter's loop).
+constexpr int PAD_NONE = 0, PAD_SAME = 1, PAD_CELL = 2;
+
 // ---------------------------------------------------------------- errors
 struct Error {
   paw_status code;
@@ -229,8 +234,7 @@ struct paw_context {
   // and the scalar images of the block (FP64 -Lambda, Lambda_Y, alpha Lambda_Y;
   // FP32 hi/lo words)
   pawfe::DevBuf ws_Y0p[2], ws_lamp[2], ws_cfp[2];
-  int lean = 0;      // 1: persistent cell/projection kernels in their half-shared-memory form
-  int sf_lean = 0;   // 1: FP64 sum-factorised kernel in its 4-vector form
+  int padded = 0;    // PAD_*: work on a block padded to whole 16-byte rows is being issued
   cudaStream_t s_loop = nullptr, s_side = nullptr;   // internal streams of the overlapped filter
   std::vector<cudaEvent_t> ev_pool;
   size_t ev_used = 0;
@@ -389,7 +393,8 @@ struct ChebScalars {
 size_t cheb_nd(int nb, int m);
 size_t cheb_nf(int nb, int m);
 void cheb_plan(int nb, int m, paw_bounds bd, const double *lam, ChebScalars &S, double *hd, float *hf);
-void cheb_issue(paw_context *c, paw_precision prec, const double *X, int ldx, int nb, paw_bounds bd,
+// nbp >= nb: columns that the loop works on (the images are planned for nbp).
+void cheb_issue(paw_context *c, paw_precision prec, const double *X, int ldx, int nb, int nbp, paw_bounds bd,
                 const ChebScalars &S, const double *hd, const float *hf, double *Xo, int ldo, cudaStream_t s,
                 const double *hd_dev = nullptr, const float *hf_dev = nullptr);
 

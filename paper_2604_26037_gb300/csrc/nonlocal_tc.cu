@@ -489,22 +489,28 @@ __global__ void k_build_expB(const float *__restrict__ oP, const int *__restrict
 
 // ------------------------------------------------------------------ streaming forms
 // Persistent warp-specialised forms (tc_stream.cuh) for 16-byte-aligned rows.
-// LEAN: two stages, the form used while an FP64 step 2 shares the SMs.
-template <bool LEAN = false>
+// SC: the rows are multiplied by M_D^-1 before they are rounded (as in k_nl_project_tc, for
+// padded blocks) instead of with the images that hold M_D^-1 P.
+template <bool SC>
 struct ProjStream {
-  static constexpr int NW = 1, S = LEAN ? 2 : 4, NEPI = 4;
-  static constexpr bool BF16 = false;
+  static constexpr int S = 4, NEPI = 4;
+  static constexpr bool BF16 = false, TRUNC = false, SCALED = SC;
   static constexpr uint32_t B_MAX = 192u * 128u;
-  CUtensorMap tm[NW];   // rows of X (gathered with TMA)
+  CUtensorMap tm;       // rows of X (gathered with TMA)
   int ntiles, ncols, n, p, N1, own, npad, kc_own, ppt, vtiles, ldx;
   const int *own_off, *own_atom;
   const uint8_t *B;
   const float *X;
   float *U;             // per-atom sums (zeroed before the launch)
+  const float *mdo;     // M_D^-1 in owner order, ostride entries per cell
+  int ostride;
   struct Tile {
     int e, vt, k0, np;
     int64_t cb;
   };
+  __device__ float row_scale(const Tile &T, int kc, int j) const {
+    return __ldg(mdo + (size_t)T.e * ostride + min(kc * 32 + j, own - 1));
+  }
   __device__ Tile tile(int t) const {
     Tile T;
     T.e = t / vtiles;
@@ -519,14 +525,13 @@ struct ProjStream {
   __device__ int nchunks(const Tile &, int) const { return kc_own; }
   __device__ int ncol(const Tile &T, int sub) const { return min(ppt, T.np - sub * ppt) * npad; }
   __device__ int xcol(const Tile &T) const { return T.vt * MT; }
-  __device__ int row_id(const Tile &T, int, int kc, int j, int) const {
+  __device__ int row_id(const Tile &T, int, int kc, int j) const {
     const int o = kc * 32 + j;
     return o < own ? (int)(T.cb + owned_offset(o, p, N1)) : -1;
   }
   __device__ const uint8_t *bsrc(const Tile &T, int sub, int kc) const {
     return B + (size_t)(T.k0 + sub * ppt) * npad * 128 * kc_own + (size_t)kc * ncol(T, sub) * 128;
   }
-  __device__ uint32_t dcol(int) const { return 0; }
   // U[atom of pair][al][v] += column (pair, al) of the tile: FP32 reductions into
   // the per-atom sums (no per-pair partials); four warps, one per lane quarter.
   // Columns come in whole pairs of npad (a multiple of 16), so a 16-column
@@ -1026,9 +1031,6 @@ template <class P>
 static void launch_stream(const paw_context *c, const P &p, cudaStream_t s, const char *what) {
   const size_t shm = tcs::Geo<P>::SMEM;
   PAW_CUDA(cudaFuncSetAttribute(tcs::k_tc_stream<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
-  if (c->lean)   // the whole shared memory configured, so that an FP64 CTA fits beside this one
-    PAW_CUDA(cudaFuncSetAttribute(tcs::k_tc_stream<P>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                  cudaSharedmemCarveoutMaxShared));
   const int grid = std::max(1, std::min(p.ntiles, persistent_grid(c)));
   tcs::k_tc_stream<P><<<grid, tcs::threads_for(P::NEPI), shm, s>>>(p, c->status_dev.as<int>(), c->wait_ns,
                                                                      c->wait_probe);
@@ -1039,11 +1041,11 @@ static bool rows16(const void *p, int ld) {
   return reinterpret_cast<uintptr_t>(p) % 16 == 0 && ld % 4 == 0;
 }
 
-template <bool LEAN>
+template <bool SC>
 static void proj_stream(paw_context *c, const float *X, int ldx, int ncols, bool scaled, float *U, int vtiles,
                         cudaStream_t s) {
   const NlTcMats &N = c->nltc;
-  ProjStream<LEAN> p;
+  ProjStream<SC> p;
   p.ntiles = c->ncells * vtiles;
   p.ncols = ncols;
   p.n = c->n;
@@ -1057,12 +1059,14 @@ static void proj_stream(paw_context *c, const float *X, int ldx, int ncols, bool
   p.ldx = ldx;
   p.own_off = c->own_off.as<int>();
   p.own_atom = c->own_atom.as<int>();
-  p.B = scaled ? N.projBs.as<uint8_t>() : N.projB.as<uint8_t>();
+  p.B = scaled && !SC ? N.projBs.as<uint8_t>() : N.projB.as<uint8_t>();
   p.X = X;
   p.U = U;
+  p.mdo = N.mdo.as<float>();
+  p.ostride = N.nh * N.ntile;
   PAW_CUDA(cudaMemsetAsync(U, 0, sizeof(float) * (size_t)c->natoms * c->npad * ncols, s));
-  encode_row_map(&p.tm[0], X, c->ndof, ncols, ldx);
-  launch_stream(c, p, s, LEAN ? "k_tc_stream<projection, lean>" : "k_tc_stream<projection>");
+  encode_row_map(&p.tm, X, c->ndof, ncols, ldx);
+  launch_stream(c, p, s, "k_tc_stream<projection>");
 }
 
 bool nltc_project(paw_context *c, const float *X, int ldx, int ncols, const float *rowscale, float *PP,
@@ -1073,7 +1077,7 @@ bool nltc_project(paw_context *c, const float *X, int ldx, int ncols, const floa
   const int vtiles = (ncols + MT - 1) / MT;
   const bool scaled = rowscale != nullptr && rowscale == c->md_inv32.as<float>();
   if (c->tc_variant == 0 && (rowscale == nullptr || scaled) && rows16(X, ldx) && ncols % 4 == 0) {
-    if (c->lean)
+    if (c->padded == PAD_SAME && scaled)
       proj_stream<true>(c, X, ldx, ncols, scaled, U, vtiles, s);
     else
       proj_stream<false>(c, X, ldx, ncols, scaled, U, vtiles, s);
@@ -1144,8 +1148,6 @@ static void expand_stream(paw_context *c, const ExpArgs &A, const float *W1, con
       encode_row_map(&p.tm[k], static_cast<const float *>(arr[k]), c->ndof, A.ncols, ld[k]);
       p.amask |= 1 << k;
     }
-  // (the expansion keeps its four staged groups while a step 2 shares the SMs: a two-group
-  // form, 160 KB, still leaves too little room for the FP64 kernel and slowed the loop)
   const size_t shm = xs::smem_bytes<MODE>();
   PAW_CUDA(cudaFuncSetAttribute(xs::k_exp_stream<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
   const int grid = std::max(1, std::min(p.ntiles, persistent_grid(c)));

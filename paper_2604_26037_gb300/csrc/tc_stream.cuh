@@ -5,7 +5,10 @@
 // A tile is one or more accumulation rounds
 //     D (128 vectors x N) = A (128 vectors x K) . B (N x K)^T
 // into a double-buffered FP32 accumulator in tensor memory (2 x 256 columns),
-// so the epilogue of one round overlaps the MMAs of the next.
+// so the epilogue of one round overlaps the MMAs of the next.  (Two such products of 256
+// vectors with one landed B, into a single buffer of 2 x 256 columns, land 29% fewer bytes per
+// vector but leave shared memory for two stages and no overlap of the epilogue: cell products
+// of the mid workload 1.32 instead of 1.09 ms per step.)
 //
 // The rows of A are contiguous 128-vector slices of a row-major block (a node
 // row of a DoF-major multivector, or a projector row of the atom-major
@@ -80,12 +83,12 @@ template <class P>
 struct Geo {
   static constexpr int KR = P::BF16 ? 64 : 32;                  // A rows (K elements) per chunk
   static constexpr uint32_t RAW = KR * ROW_BYTES;               // raw rows of one operand
-  static constexpr uint32_t STAGE = P::NW * (RAW + A_BYTES) + P::B_MAX;
+  static constexpr uint32_t STAGE = RAW + A_BYTES + P::B_MAX;
   // at least 120 KB: one CTA per SM, so that its 512 TMEM columns are always free
   static constexpr size_t SMEM0 = 1024 + (size_t)P::S * STAGE + sizeof(Shared);
   static constexpr size_t SMEM = SMEM0 < 120 * 1024 ? 120 * 1024 : SMEM0;
   static_assert(P::B_MAX % 1024 == 0, "B stage must keep 1024-byte alignment");
-  static_assert(P::S >= 2 && P::S <= SMAX && P::NW >= 1 && P::NW <= 2, "stage / operand counts");
+  static_assert(P::S >= 2 && P::S <= SMAX, "stage count");
   static_assert(P::NEPI % 4 == 0, "epilogue warps come in lane-quarter groups");
 };
 
@@ -119,16 +122,16 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatil
 }
 
 template <class P>
-__device__ __forceinline__ uint8_t *stage_raw(uint8_t *base, int s, int w) {
-  return base + (size_t)s * Geo<P>::STAGE + (size_t)w * Geo<P>::RAW;
+__device__ __forceinline__ uint8_t *stage_raw(uint8_t *base, int s) {
+  return base + (size_t)s * Geo<P>::STAGE;
 }
 template <class P>
-__device__ __forceinline__ uint8_t *stage_A(uint8_t *base, int s, int w) {
-  return base + (size_t)s * Geo<P>::STAGE + (size_t)P::NW * Geo<P>::RAW + (size_t)w * A_BYTES;
+__device__ __forceinline__ uint8_t *stage_A(uint8_t *base, int s) {
+  return base + (size_t)s * Geo<P>::STAGE + Geo<P>::RAW;
 }
 template <class P>
 __device__ __forceinline__ uint8_t *stage_B(uint8_t *base, int s) {
-  return base + (size_t)s * Geo<P>::STAGE + (size_t)P::NW * (Geo<P>::RAW + A_BYTES);
+  return base + (size_t)s * Geo<P>::STAGE + Geo<P>::RAW + A_BYTES;
 }
 
 // ------------------------------------------------------------------ roles
@@ -171,11 +174,9 @@ struct Walk {
 
 // row indices of the current chunk: lane l holds rows l, 32 + l, ... (-1: no row)
 template <class P>
-__device__ __forceinline__ void chunk_ids(const P &p, const Walk<P> &w, int lane, int (&rid)[P::NW][Geo<P>::KR / 32]) {
+__device__ __forceinline__ void chunk_ids(const P &p, const Walk<P> &w, int lane, int (&rid)[Geo<P>::KR / 32]) {
 #pragma unroll
-  for (int o = 0; o < P::NW; ++o)
-#pragma unroll
-    for (int jj = 0; jj < Geo<P>::KR / 32; ++jj) rid[o][jj] = p.row_id(w.T, w.sub, w.kc, jj * 32 + lane, o);
+  for (int jj = 0; jj < Geo<P>::KR / 32; ++jj) rid[jj] = p.row_id(w.T, w.sub, w.kc, jj * 32 + lane);
 }
 
 template <class P>
@@ -186,7 +187,7 @@ __device__ void role_loader(const P &p, uint8_t *base, Shared *sh, int lane) {
   bool run = __shfl_sync(0xffffffffu, *abort, 0) == 0;   // warp-uniform
   Walk<P> w;
   bool have = w.start(p);
-  int rid[P::NW][RPL];
+  int rid[RPL];
   if (have) chunk_ids<P>(p, w, lane, rid);
   for (; run && have; ++g) {
     const int s = (int)(g % S);
@@ -197,31 +198,27 @@ __device__ void role_loader(const P &p, uint8_t *base, Shared *sh, int lane) {
     }
     const uint32_t full = smem_u32(&sh->full[s]);
     const uint32_t bbytes = (uint32_t)p.ncol(w.T, w.sub) * 128u;
-    if (lane == 0) mbar_arrive_tx(full, bbytes + (uint32_t)(P::NW * KR) * ROW_BYTES);
+    if (lane == 0) mbar_arrive_tx(full, bbytes + (uint32_t)KR * ROW_BYTES);
     __syncwarp();
     if (lane == 0) bulk_g2s(smem_u32(stage_B<P>(base, s)), p.bsrc(w.T, w.sub, w.kc), bbytes, full);
-    const int x = p.xcol(w.T);
+    // rows that do not exist repeat the chunk's first row (always present)
+    const int first = __shfl_sync(0xffffffffu, rid[0], 0);
+    // lane l < KR / 4 gathers rows 4 l .. 4 l + 3, held by lanes (4 l + i) % 32, slot (4 l + i) / 32
+    int r4[4];
 #pragma unroll
-    for (int o = 0; o < P::NW; ++o) {
-      // rows that do not exist repeat the chunk's first row (always present)
-      const int first = __shfl_sync(0xffffffffu, rid[o][0], 0);
-      // lane l < KR / 4 gathers rows 4 l .. 4 l + 3, held by lanes (4 l + i) % 32, slot (4 l + i) / 32
-      int r4[4];
+    for (int i = 0; i < 4; ++i) {
+      const int row = 4 * lane + i;
+      int val = 0;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int row = 4 * lane + i;
-        int val = 0;
-#pragma unroll
-        for (int jj = 0; jj < RPL; ++jj) {
-          const int t = __shfl_sync(0xffffffffu, rid[o][jj], row & 31);
-          if ((row >> 5) == jj) val = t;
-        }
-        r4[i] = val >= 0 ? val : first;
+      for (int jj = 0; jj < RPL; ++jj) {
+        const int t = __shfl_sync(0xffffffffu, rid[jj], row & 31);
+        if ((row >> 5) == jj) val = t;
       }
-      if (lane < KR / 4)
-        tma_gather4(smem_u32(stage_raw<P>(base, s, o)) + (uint32_t)lane * 4u * ROW_BYTES, &p.tm[o], x, r4[0], r4[1],
-                    r4[2], r4[3], full);
+      r4[i] = val >= 0 ? val : first;
     }
+    if (lane < KR / 4)
+      tma_gather4(smem_u32(stage_raw<P>(base, s)) + (uint32_t)lane * 4u * ROW_BYTES, &p.tm, p.xcol(w.T), r4[0], r4[1],
+                  r4[2], r4[3], full);
     have = w.next(p);
     if (have) chunk_ids<P>(p, w, lane, rid);   // consumed after the next stage wait
   }
@@ -255,33 +252,33 @@ __device__ void role_transpose(const P &p, uint8_t *base, Shared *sh, int r) {
           run = false;
           break;
         }
+        const float *raw = reinterpret_cast<const float *>(stage_raw<P>(base, s));
+        uint8_t *A = stage_A<P>(base, s);
 #pragma unroll
-        for (int w = 0; w < P::NW; ++w) {
-          const float *raw = reinterpret_cast<const float *>(stage_raw<P>(base, s, w));
-          uint8_t *A = stage_A<P>(base, s, w);
+        for (int c = 0; c < 8; ++c) {
+          uint4 q;
+          if constexpr (P::BF16) {
+            uint32_t h[4];
 #pragma unroll
-          for (int c = 0; c < 8; ++c) {
-            uint4 q;
-            if constexpr (P::BF16) {
-              uint32_t h[4];
-#pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                const int j = c * 8 + 2 * i;
-                __nv_bfloat162 b2 = __floats2bfloat162_rn(raw[j * MT + r], raw[(j + 1) * MT + r]);
-                h[i] = *reinterpret_cast<uint32_t *>(&b2);
-              }
-              q = make_uint4(h[0], h[1], h[2], h[3]);
-            } else {
-              uint32_t h[4];
-#pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                const int j = c * 4 + i;
-                h[i] = to_tf32(raw[j * MT + r]);
-              }
-              q = make_uint4(h[0], h[1], h[2], h[3]);
+            for (int i = 0; i < 4; ++i) {
+              const int j = c * 8 + 2 * i;
+              __nv_bfloat162 b2 = __floats2bfloat162_rn(raw[j * MT + r], raw[(j + 1) * MT + r]);
+              h[i] = *reinterpret_cast<uint32_t *>(&b2);
             }
-            *reinterpret_cast<uint4 *>(A + sw128_off(r, c)) = q;
+            q = make_uint4(h[0], h[1], h[2], h[3]);
+          } else {
+            uint32_t h[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const int j = c * 4 + i;
+              float x = raw[j * MT + r];
+              if constexpr (P::SCALED) x = __fmul_rn(x, p.row_scale(T, kc, j));
+              // (P::TRUNC: the tensor core takes the TF32 part of the FP32 number)
+              h[i] = P::TRUNC ? __float_as_uint(x) : to_tf32(x);
+            }
+            q = make_uint4(h[0], h[1], h[2], h[3]);
           }
+          *reinterpret_cast<uint4 *>(A + sw128_off(r, c)) = q;
         }
         fence_proxy_async();
         mbar_arrive(smem_u32(&sh->afull[s]));
@@ -318,14 +315,11 @@ __device__ void role_mma(const P &p, uint8_t *base, Shared *sh, uint32_t tmem) {
         }
         tc_fence_after();
         const uint64_t bd = sw128_desc(smem_u32(stage_B<P>(base, s)));
+        const uint64_t ad = sw128_desc(smem_u32(stage_A<P>(base, s)));
 #pragma unroll
-        for (int w = 0; w < P::NW; ++w) {
-          const uint64_t ad = sw128_desc(smem_u32(stage_A<P>(base, s, w)));
-#pragma unroll
-          for (int j = 0; j < 4; ++j)   // K-step j: 32 bytes of every K-major row
-            mma<P::BF16>(tmem + (uint32_t)(b * 256) + p.dcol(w), ad + (uint64_t)(2 * j), bd + (uint64_t)(2 * j),
-                         idesc, (kc | j) != 0);
-        }
+        for (int j = 0; j < 4; ++j)   // K-step j: 32 bytes of every K-major row
+          mma<P::BF16>(tmem + (uint32_t)(b * 256), ad + (uint64_t)(2 * j), bd + (uint64_t)(2 * j), idesc,
+                       (kc | j) != 0);
         mma_commit(smem_u32(&sh->empty[s]));
       }
       if (!run) break;
