@@ -263,30 +263,26 @@ static void merge_cplx(paw_context *c, const T *Xs, int n, T *Z, int ldz, cudaSt
 // Y = H X - S X Lambda in FP64 (Algorithm 2 step 2)
 static void residual_block(paw_context *c, const double *X, int ldx, const double *negLam_dev,
                            double *Y, int ldy, int ncols, cudaStream_t s, int nzero = 0) {
-  zero_block<double>(Y, c->ndof, std::max(ncols, nzero), ldy, s);   // (columns past ncols stay zero)
-  // both parts add into Y (the local part first: with the nonlocal part first beside a
-  // loop, the mid filter call measured 293 instead of 288 ms)
-  auto nonlocal = [&]() {
-    if (c->nown_pairs > 0) {
-      PhaseScope ps(c, 4, s);
-      // sum_a P^a (D_H^a - lambda_j dS^a) P^a^T x_j: one projection, one expansion
-      c->scr->W2.ensure(sizeof(double) * (size_t)c->natoms * c->npad * ncols, &c->dev_bytes);
-      double *W = c->scr->W2.as<double>();
-      nl_project_residual<double>(c, X, ldx, ncols, negLam_dev, W, s);
-      nl_expand<double>(c, PAW_FP64, W, ncols, Y, ldy, nullptr, s);
-    }
-  };
+  // the nonlocal part writes every row of the ncols columns, then the local part adds into them
+  if (nzero > ncols) zero_block<double>(Y + ncols, c->ndof, nzero - ncols, ldy, s);
+  if (c->nown_pairs > 0) {
+    PhaseScope ps(c, 4, s);
+    // sum_a P^a (D_H^a - lambda_j dS^a) P^a^T x_j: one projection, one expansion
+    c->scr->W2.ensure(sizeof(double) * (size_t)c->natoms * c->npad * ncols, &c->dev_bytes);
+    double *W = c->scr->W2.as<double>();
+    nl_project_residual<double>(c, X, ldx, ncols, negLam_dev, W, s);
+    nl_expand<double>(c, PAW_FP64, W, ncols, Y, ldy, s);
+  } else {
+    zero_block<double>(Y, c->ndof, ncols, ldy, s);
+  }
   // (1/2 K^e + V^e + (1/2 |k|^2 - lambda_j) M^e) X_e in one sum-factorised pass;
   // at k != 0 the Bloch term -i B of Eq. hij on the split block [Re | Im]
-  {
-    PhaseScope ps(c, 0, s);
-    local_sf(c, X, ldx, Y, ldy, ncols, 1.0, 1.0, 1.0, c->kmass, negLam_dev, s);
-    if (c->kc) {
-      bloch_sf(c, X + ncols / 2, ldx, Y, ldy, ncols / 2, 1.0, s);
-      bloch_sf(c, X, ldx, Y + ncols / 2, ldy, ncols / 2, -1.0, s);
-    }
+  PhaseScope ps(c, 0, s);
+  local_sf(c, X, ldx, Y, ldy, ncols, 1.0, 1.0, 1.0, c->kmass, negLam_dev, s);
+  if (c->kc) {
+    bloch_sf(c, X + ncols / 2, ldx, Y, ldy, ncols / 2, 1.0, s);
+    bloch_sf(c, X, ldx, Y + ncols / 2, ldy, ncols / 2, -1.0, s);
   }
-  nonlocal();
 }
 
 template <typename T>

@@ -282,10 +282,9 @@ void cell_apply_simt(paw_context *c, const T *mats, long long stride, const T *X
 template <typename T>
 void nl_project(paw_context *c, paw_precision prec, const T *X, int ldx, int ncols, const T *rowscale,
                 const double *coup, double coup_scale, T *W, cudaStream_t s);
-// Y[dof] += colscale[j] * sum_a P^a W[a]   (owner-cell expansion, no atomics)
+// Y[dof] = sum_a P^a W[a] on every DoF   (owner-cell expansion, no atomics)
 template <typename T>
-void nl_expand(paw_context *c, paw_precision prec, const T *W, int ncols, T *Y, int ldy,
-               const double *colscale, cudaStream_t s);
+void nl_expand(paw_context *c, paw_precision prec, const T *W, int ncols, T *Y, int ldy, cudaStream_t s);
 // Y = M_D^-1 (X - sum_a P^a W[a])
 template <typename T>
 void nl_sinv_out(paw_context *c, paw_precision prec, const T *W, int ncols, const T *X, int ldx, T *Y,
@@ -318,7 +317,7 @@ void nltc_prepare(paw_context *c, cudaStream_t s);
 // the one-CTA-per-tile form writes per-pair partials PP[k][al][v] (returns false)
 bool nltc_project(paw_context *c, const float *X, int ldx, int ncols, const float *rowscale, float *PP,
                   float *U, cudaStream_t s);
-// expansion with the output stage of mode (EXP_ADD / EXP_SINV / EXP_RECURRENCE)
+// expansion with the output stage of mode (EXP_SET / EXP_SINV / EXP_RECURRENCE)
 struct ExpArgs;
 void nltc_expand(paw_context *c, int mode, const ExpArgs &A, const float *W1, const float *W2, cudaStream_t s);
 // FP64 data (nonlocal_fx.cu): per-pair partials U[k][al][v] of P^T (rowscale .* X), and the

@@ -487,11 +487,11 @@ __global__ void __launch_bounds__(NPAD / 2 * 32) k_couple_h_c(int np, const int 
 }
 
 // ------------------------------------------------------------------ expansion
-// FP32 SIMT form (the FP64 form is k_own_expand64 below).
+// FP32 SIMT form (the FP64 form is k_fx_expand in nonlocal_fx.cu).
 // Expansion with a fused output stage.  W of every pair of the cell is staged
 // in shared memory (VT vectors of each: 32, or 4 for cells with many pairs);
 // a thread owns 4 vectors of one node row at a time.
-//   EXP_ADD        Y += cs[v] * S1
+//   EXP_SET        Y = S1 (zero in cells that no projector reaches)
 //   EXP_SINV       Y  = md_inv * (X - S1)                                         (Eq. Sinvapprox)
 //   EXP_RECURRENCE T  = md_inv * (R_Y - S1)
 //                  R_X = [-beta R_Y - gamma R_X + S2] + alpha Y Lambda_Y   (S2: nonlocal part of alpha H T)
@@ -506,7 +506,6 @@ __global__ void __launch_bounds__(256, 2) k_own_expand(ExpArgs A, const T *__res
   extern __shared__ __align__(16) unsigned char sm_raw[];
   const int e = blockIdx.y, v0 = blockIdx.x * VT;   // vector tiles of one cell are adjacent: P reused from L2
   const int k0 = A.own_off[e], k1 = A.own_off[e + 1];
-  if (MODE == EXP_ADD && k0 == k1) return;
   const int own = A.p * A.p * A.p;
   const int np = k1 - k0;
   const int ncols = A.ncols;
@@ -540,17 +539,13 @@ __global__ void __launch_bounds__(256, 2) k_own_expand(ExpArgs A, const T *__res
   // output stage of one node row o with its sums s1, s2 over the 4 vectors v .. v+3
   auto emit = [&](int o, const T (&s1)[4], const T (&s2)[4]) {
     const int64_t d = base + ooff[o];
-    if (MODE == EXP_ADD) {
+    if (MODE == EXP_SET) {
       T *yp = Y + d * A.ldy + v;
       if (vec) {
-        T y[4];
-        ld4(yp, y);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) y[j] += (A.cs ? T(A.cs[v + j]) : T(1)) * s1[j];
-        st4(yp, y);
+        st4(yp, s1);
       } else {
         for (int j = 0; j < 4; ++j)
-          if (v + j < ncols) yp[j] += (A.cs ? T(A.cs[v + j]) : T(1)) * s1[j];
+          if (v + j < ncols) yp[j] = s1[j];
       }
     } else if (MODE == EXP_SINV) {
       const T m = mdinv[d];
@@ -872,16 +867,14 @@ static ExpArgs exp_args(paw_context *c, int ncols) {
 }
 
 template <typename T>
-void nl_expand(paw_context *c, paw_precision prec, const T *W, int ncols, T *Y, int ldy, const double *colscale,
-               cudaStream_t s) {
+void nl_expand(paw_context *c, paw_precision prec, const T *W, int ncols, T *Y, int ldy, cudaStream_t s) {
   if (c->nown_pairs == 0 || ncols <= 0) return;
   ExpArgs A = exp_args(c, ncols);
   A.Y = Y;
   A.ldy = ldy;
   A.ldx = ldy;
   A.ldy0 = 4;
-  A.cs = colscale;
-  own_expand<T, EXP_ADD>(c, prec, A, W, nullptr, s);
+  own_expand<T, EXP_SET>(c, prec, A, W, nullptr, s);
 }
 
 template <typename T>
@@ -946,9 +939,9 @@ template void nl_project_filter<double>(paw_context *, paw_precision, const doub
                                         double, double *, double *, cudaStream_t);
 template void nl_project_filter<float>(paw_context *, paw_precision, const float *, int, int, const float *,
                                        double, float *, float *, cudaStream_t);
-template void nl_expand<double>(paw_context *, paw_precision, const double *, int, double *, int, const double *,
+template void nl_expand<double>(paw_context *, paw_precision, const double *, int, double *, int,
                                 cudaStream_t);
-template void nl_expand<float>(paw_context *, paw_precision, const float *, int, float *, int, const double *,
+template void nl_expand<float>(paw_context *, paw_precision, const float *, int, float *, int,
                                cudaStream_t);
 template void nl_sinv_out<double>(paw_context *, paw_precision, const double *, int, const double *, int, double *,
                                   int, const double *, cudaStream_t);

@@ -18,17 +18,16 @@ __device__ __forceinline__ float add_product_df(float b, float ch, float cl, flo
   return __fadd_rn(s, __fadd_rn(err, tl));
 }
 
-constexpr int EXP_ADD = 0, EXP_SINV = 1, EXP_RECURRENCE = 2;
+constexpr int EXP_SET = 0, EXP_SINV = 1, EXP_RECURRENCE = 2;
 
 struct ExpArgs {
   int n, p, N1;
   const int *own_off, *own_atom;
   const int *own_ngrp;           // per pair: groups of 4 projectors with nonzero values
   int ncols;
-  const double *cs;              // ADD: per-column factor (may be NULL)
   const void *Xin;               // SINV: X; RECURRENCE: R_Y
   int ldx;
-  void *Y;                       // ADD/SINV output; RECURRENCE: T
+  void *Y;                       // SET/SINV output; RECURRENCE: T
   int ldy;
   const void *mdinv;
   void *RX;                      // RECURRENCE: R_X (ld = ldx)

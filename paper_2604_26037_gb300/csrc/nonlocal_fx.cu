@@ -316,7 +316,6 @@ __global__ void __launch_bounds__(256, 2) k_fx_expand(FxNl N, ExpArgs A, const d
   const int ncols = A.ncols, ntile = (ncols + VT - 1) / VT;
   const int e = blockIdx.x / ntile, v0 = (blockIdx.x - e * ntile) * VT;
   const int k0 = N.own_off[e], np = N.own_off[e + 1] - k0;
-  if (MODE == EXP_ADD && np == 0) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, own = N.own;
   for (int o = tid; o < own; o += 256) ooff[o] = owned_offset(o, N.p, N.N1);   // (synchronised with the maxima)
   const int vp = tid % VP, r0 = tid / VP;
@@ -395,17 +394,16 @@ __global__ void __launch_bounds__(256, 2) k_fx_expand(FxNl N, ExpArgs A, const d
           }
           if (o >= own) continue;
           const int64_t d = base + ooff[o];
-          const double m = MODE == EXP_ADD ? 0.0 : static_cast<const double *>(A.mdinv)[d];
+          const double m = MODE == EXP_SET ? 0.0 : static_cast<const double *>(A.mdinv)[d];
           double *Y = static_cast<double *>(A.Y) + d * A.ldy + v0 + l0;
-          const double *Xi = MODE == EXP_ADD ? nullptr : static_cast<const double *>(A.Xin) + d * A.ldx + v0 + l0;
+          const double *Xi = MODE == EXP_SET ? nullptr : static_cast<const double *>(A.Xin) + d * A.ldx + v0 + l0;
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
             const int c = (i >> 1) * 8 + (i & 1);
             if (v0 + l0 + c >= ncols) continue;
             const long long s = t.s[i >> 1][2 * r + (i & 1)];
-            if (MODE == EXP_ADD) {
-              const double y = value(s, Em[0][l0 + c]);
-              Y[c] += y;
+            if (MODE == EXP_SET) {
+              Y[c] = value(s, Em[0][l0 + c]);
             } else if (MODE == EXP_SINV) {
               Y[c] = m * (Xi[c] - value(s, Em[0][l0 + c]));
             } else {
@@ -501,8 +499,8 @@ void launch_expand(paw_context *c, const ExpArgs &A, const double *W1, const dou
 
 template <int NPAD, int VT>
 void expand_mode(paw_context *c, int mode, const ExpArgs &A, const double *W1, const double *W2, cudaStream_t s) {
-  if (mode == EXP_ADD)
-    launch_expand<NPAD, VT, EXP_ADD>(c, A, W1, W2, s);
+  if (mode == EXP_SET)
+    launch_expand<NPAD, VT, EXP_SET>(c, A, W1, W2, s);
   else if (mode == EXP_SINV)
     launch_expand<NPAD, VT, EXP_SINV>(c, A, W1, W2, s);
   else
@@ -546,7 +544,6 @@ void nlfx_project(paw_context *c, const double *X, int ldx, int ncols, const dou
 void nlfx_expand(paw_context *c, int mode, const ExpArgs &A, const double *W1, const double *W2, cudaStream_t s) {
   PAW_REQUIRE(c->max_own_pairs <= PAIRS_PER_CELL_MAX && c->own <= 512, PAW_ERR_UNSUPPORTED,
               "too many atoms on one cell for the expansion kernel");
-  PAW_REQUIRE(!A.cs, PAW_ERR_UNSUPPORTED, "the FP64 expansion has no column factors");
   const bool narrow = A.ncols <= 16 || expand_smem(c, mode, 32) > FX_SMEM_MAX;
   if (c->npad == 16)
     narrow ? expand_mode<16, 16>(c, mode, A, W1, W2, s) : expand_mode<16, 32>(c, mode, A, W1, W2, s);

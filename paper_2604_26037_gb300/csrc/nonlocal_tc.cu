@@ -233,7 +233,6 @@ __global__ void __launch_bounds__(THREADS, 2) k_nl_expand_tc(ExpArgs A, ExpTcArg
   const int e = bid / (a.vtiles * a.nh);
   const int k0 = A.own_off[e], k1 = A.own_off[e + 1];
   const int np = k1 - k0;
-  if (MODE == EXP_ADD && np == 0) return;   // nothing to add (uniform, before any barrier)
   if (*reinterpret_cast<volatile int *>(a.status) != 0) return;   // an earlier CTA gave up
   const int KC = a.eoff[e + 1] - a.eoff[e];
   const int ncols = A.ncols;
@@ -332,12 +331,11 @@ __global__ void __launch_bounds__(THREADS, 2) k_nl_expand_tc(ExpArgs A, ExpTcArg
     const bool wok = vout < ncols;
     const int vj = min(vout, ncols - 1);
     const uint32_t tl = tmem + ((uint32_t)(q * 32) << 16);
-    float chi = 0.f, clo = 0.f, csv = 1.f;
+    float chi = 0.f, clo = 0.f;
     if (MODE == EXP_RECURRENCE) {
       chi = A.chi[vj];
       clo = A.clo[vj];
     }
-    if (MODE == EXP_ADD && A.cs) csv = (float)A.cs[vj];
     const float *mdinv = static_cast<const float *>(A.mdinv);
     const float *Xin = static_cast<const float *>(A.Xin);
     float *Y = static_cast<float *>(A.Y);
@@ -361,16 +359,7 @@ __global__ void __launch_bounds__(THREADS, 2) k_nl_expand_tc(ExpArgs A, ExpTcArg
       // two batches of 8 node rows: all loads of a batch in flight before its stores
 #pragma unroll
       for (int jb = 0; jb < 16; jb += 8) {
-        if (MODE == EXP_ADD) {
-          float y[8];
-#pragma unroll
-          for (int j = 0; j < 8; ++j)
-            if (jb + j < nrow) y[j] = Y[(cb + ooff[c0 + jb + j]) * A.ldy + vout];
-#pragma unroll
-          for (int j = 0; j < 8; ++j)
-            if (jb + j < nrow)
-              Y[(cb + ooff[c0 + jb + j]) * A.ldy + vout] = fmaf(csv, __uint_as_float(s1[jb + j]), y[j]);
-        } else if (MODE == EXP_SINV) {
+        if (MODE == EXP_SINV) {
           float x[8], m[8];
 #pragma unroll
           for (int j = 0; j < 8; ++j)
@@ -578,7 +567,7 @@ template <int MODE>
 struct Geo {
   static constexpr int NW = (MODE == EXP_RECURRENCE) ? 2 : 1;
   static constexpr int S = (MODE == EXP_RECURRENCE) ? 2 : 3;    // A/B stages
-  static constexpr int NA = (MODE == EXP_RECURRENCE) ? 4 : 1;   // staged arrays
+  static constexpr int NA = (MODE == EXP_RECURRENCE) ? 4 : MODE == EXP_SINV ? 1 : 0;   // staged arrays
   static constexpr uint32_t STAGE = NW * A_BYTES + 128u * 128u;
   static constexpr uint32_t GROUP = NA * 16u * ROWB;              // 16 staged rows of each array
 };
@@ -598,7 +587,7 @@ constexpr size_t smem_bytes() {
 }
 
 struct Args {
-  CUtensorMap tm[4];   // staged arrays (R_Y, R_X, Y hi, Y lo; or X; or Y), rows gathered with TMA
+  CUtensorMap tm[4];   // staged arrays (R_Y, R_X, Y hi, Y lo; or X; none), rows gathered with TMA
   int amask;           // bit k: array k is staged
   ExpArgs A;
   int ntiles, npad, ppc, ntile, nh, vtiles, own;
@@ -628,11 +617,6 @@ __device__ __forceinline__ Tile tile_of(const Args &a, int t) {
   T.nrows = min(a.ntile, a.own - T.o_beg);
   T.ngroups = (T.nrows + 15) / 16;
   return T;
-}
-
-template <int MODE>
-__device__ __forceinline__ bool skip_tile(const Tile &T) {
-  return MODE == EXP_ADD && T.np == 0;   // nothing to add
 }
 
 template <int MODE>
@@ -683,7 +667,6 @@ __global__ void __launch_bounds__(THREADS, 1) k_exp_stream(const __grid_constant
       bool run = !*abort;
       for (int t = blockIdx.x; run && t < a.ntiles; t += gridDim.x) {
         const Tile T = tile_of(a, t);
-        if (skip_tile<MODE>(T)) continue;
         for (int kc = 0; kc < T.kc; ++kc, ++g) {
           const int s = (int)(g % S);
           const uint32_t u = g / S;
@@ -711,7 +694,6 @@ __global__ void __launch_bounds__(THREADS, 1) k_exp_stream(const __grid_constant
       bool run = !*abort;
       for (int t = blockIdx.x; run && t < a.ntiles; t += gridDim.x) {
         const Tile T = tile_of(a, t);
-        if (skip_tile<MODE>(T)) continue;
         const int b = (int)(tc & 1u);
         if (tc >= 2 && !tcs::wait_or_abort(smem_u32(&sh->acce[b]), ((tc >> 1) - 1) & 1u, abort)) break;
         tc_fence_after();
@@ -751,7 +733,6 @@ __global__ void __launch_bounds__(THREADS, 1) k_exp_stream(const __grid_constant
     bool run = !*abort;
     for (int t = blockIdx.x; run && t < a.ntiles; t += gridDim.x) {
       const Tile T = tile_of(a, t);
-      if (skip_tile<MODE>(T)) continue;
       const int v = T.vt * MT + r;
       const bool vok = v < ncols;
       for (int kc = 0; kc < T.kc; ++kc, ++g) {
@@ -798,9 +779,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_exp_stream(const __grid_constant
     const bool mine = k < G::NA && ((a.amask >> k) & 1);
     uint32_t gc = 0;
     bool run = __shfl_sync(0xffffffffu, *abort, 0) == 0;
-    for (int t = blockIdx.x; run && t < a.ntiles; t += gridDim.x) {
+    for (int t = blockIdx.x; G::NA > 0 && run && t < a.ntiles; t += gridDim.x) {
       const Tile T = tile_of(a, t);
-      if (skip_tile<MODE>(T)) continue;
       const int x = T.vt * MT;
       for (int gi = 0; gi < T.ngroups; ++gi, ++gc) {
         const int gb = (int)(gc % NBUF);
@@ -844,7 +824,6 @@ __global__ void __launch_bounds__(THREADS, 1) k_exp_stream(const __grid_constant
     bool run = __shfl_sync(0xffffffffu, *abort, 0) == 0;
     for (int t = blockIdx.x; run && t < a.ntiles; t += gridDim.x) {
       const Tile T = tile_of(a, t);
-      if (skip_tile<MODE>(T)) continue;
       const int b = (int)(tc & 1u);
       if (!tcs::warp_wait(smem_u32(&sh->accf[b]), (tc >> 1) & 1u, abort, lane)) break;
       tc_fence_after();
@@ -852,12 +831,11 @@ __global__ void __launch_bounds__(THREADS, 1) k_exp_stream(const __grid_constant
       const int v = T.vt * MT + vl;
       const bool vok = v < ncols;
       const int vj = min(v, ncols - 1);
-      float chi = 0.f, clo = 0.f, csv = 1.f;
+      float chi = 0.f, clo = 0.f;
       if (MODE == EXP_RECURRENCE) {
         chi = a.A.chi[vj];
         clo = a.A.clo[vj];
       }
-      if (MODE == EXP_ADD && a.A.cs) csv = (float)a.A.cs[vj];
       const uint32_t tl = tmem + (uint32_t)(b * 256) + ((uint32_t)(q * 32) << 16);
       for (int gi = 0; gi < T.ngroups; ++gi, ++gc) {
         const int gb = (int)(gc % NBUF);
@@ -868,10 +846,10 @@ __global__ void __launch_bounds__(THREADS, 1) k_exp_stream(const __grid_constant
         int dj[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-          mj[j] = (MODE != EXP_ADD) ? __ldg(a.mdo + oo + j) : 0.f;
+          mj[j] = (MODE != EXP_SET) ? __ldg(a.mdo + oo + j) : 0.f;
           dj[j] = __ldg(a.odof + oo + j);
         }
-        if (!tcs::warp_wait(smem_u32(&sh->sfull[gb]), (gc / NBUF) & 1u, abort, lane)) {
+        if (G::NA > 0 && !tcs::warp_wait(smem_u32(&sh->sfull[gb]), (gc / NBUF) & 1u, abort, lane)) {
           run = false;
           break;
         }
@@ -904,12 +882,12 @@ __global__ void __launch_bounds__(THREADS, 1) k_exp_stream(const __grid_constant
             } else if (MODE == EXP_SINV) {
               Y[d * a.A.ldy + v] = mj[j] * (sg[jr * MT + vl] - __uint_as_float(s1[j]));
             } else {
-              Y[d * a.A.ldy + v] = fmaf(csv, __uint_as_float(s1[j]), sg[jr * MT + vl]);
+              Y[d * a.A.ldy + v] = __uint_as_float(s1[j]);
             }
           }
         }
         __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&sh->sempty[gb]));
+        if (G::NA > 0 && lane == 0) mbar_arrive(smem_u32(&sh->sempty[gb]));
       }
       if (!run) break;
       tc_fence_before();
@@ -1129,7 +1107,7 @@ static void expand_stream(paw_context *c, const ExpArgs &A, const float *W1, con
   p.W2 = W2;
   p.mdo = N.mdo.as<float>();
   p.odof = N.odof.as<int>();
-  // staged arrays: R_Y, R_X, Y hi, Y lo (recurrence); X (Shat^-1); Y (add)
+  // staged arrays: R_Y, R_X, Y hi, Y lo (recurrence); X (Shat^-1)
   const void *arr[4] = {nullptr, nullptr, nullptr, nullptr};
   int ld[4] = {0, 0, 0, 0};
   if (MODE == EXP_RECURRENCE) {
@@ -1139,8 +1117,6 @@ static void expand_stream(paw_context *c, const ExpArgs &A, const float *W1, con
     arr[3] = A.Y0lo, ld[3] = A.ldy0;
   } else if (MODE == EXP_SINV) {
     arr[0] = A.Xin, ld[0] = A.ldx;
-  } else {
-    arr[0] = A.Y, ld[0] = A.ldy;
   }
   p.amask = 0;
   for (int k = 0; k < 4; ++k)
@@ -1167,10 +1143,10 @@ void nltc_expand(paw_context *c, int mode, const ExpArgs &A, const float *W1, co
   else if (mode == EXP_SINV)
     rows_ok = rows_ok && rows16(A.Xin, A.ldx);
   else
-    rows_ok = rows_ok && rows16(A.Y, A.ldy);
+    rows_ok = true;   // no operand is copied
   if (rows_ok) {
-    if (mode == EXP_ADD)
-      expand_stream<EXP_ADD>(c, A, W1, W2, s);
+    if (mode == EXP_SET)
+      expand_stream<EXP_SET>(c, A, W1, W2, s);
     else if (mode == EXP_SINV)
       expand_stream<EXP_SINV>(c, A, W1, W2, s);
     else
@@ -1191,10 +1167,6 @@ void nltc_expand(paw_context *c, int mode, const ExpArgs &A, const float *W1, co
   PAW_REQUIRE(blocks < (1ll << 31), PAW_ERR_UNSUPPORTED, "too many expansion tiles");
   const size_t shm = exp_smem(mode == EXP_RECURRENCE ? 2 : 1);
   switch (mode) {
-    case EXP_ADD:
-      PAW_CUDA(cudaFuncSetAttribute(k_nl_expand_tc<EXP_ADD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
-      k_nl_expand_tc<EXP_ADD><<<(unsigned)blocks, THREADS, shm, s>>>(A, a, W1, W2);
-      break;
     case EXP_SINV:
       PAW_CUDA(
           cudaFuncSetAttribute(k_nl_expand_tc<EXP_SINV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
