@@ -6,6 +6,7 @@
 #include <cusolverDn.h>
 
 #include <cstdint>
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -23,6 +24,8 @@ constexpr int PAIRS_PER_CELL_MAX = 192;
 constexpr int PAD_NONE = 0, PAD_SAME = 1, PAD_CELL = 2;
 
 // ---------------------------------------------------------------- errors
+struct SfPlans;
+
 struct Error {
   paw_status code;
   std::string msg;
@@ -185,6 +188,7 @@ struct paw_context {
   pawfe::DevBuf Vq;                           // ncells*nq
   pawfe::DevBuf wV;                           // ncells*nq: w_q detJ V_q in fixed point (sum-factorised V^e)
   int wV_valid = 0;
+  std::shared_ptr<pawfe::SfPlans> sf_plans;   // fixed-point tables of the FP64 operators (sumfac.cu)
   pawfe::DevBuf wVs;                          // ncells: exponents of wV's fixed-point numbers
   pawfe::TcMats tc_tf32, tc_bf16;
   pawfe::TcMats tc_bk_tf32, tc_bk_bf16;       // tcgen05 images of B^e (one shared matrix)

@@ -16,6 +16,7 @@
 // SM.  All FP64 paths (Y = H X - S X Lambda, the FP64 filter form, Rayleigh-Ritz
 // products, residuals) use this form.
 #include <algorithm>
+#include <memory>
 #include <type_traits>
 #include <vector>
 
@@ -719,31 +720,144 @@ void with_sizes(const paw_context *c, int ncols, const char *what, F f) {
 
 }  // namespace
 
+// Tables of a handle in fixed point, kept between calls (they depend on the mesh and on the
+// factors of the call, not on its vectors): making them takes the host longer than a small
+// application takes the GPU.  A bounded number, the oldest is replaced.
+struct SfPlans {
+  static constexpr size_t MAX = 4;
+  Tab1 M, D, C, phi, pht;
+  struct Local {
+    double alpha, cK, cV, cM;
+    FxLocal t;
+  };
+  struct Bloch {
+    double alpha;
+    FxBloch t;
+  };
+  std::vector<Local> local;
+  std::vector<Bloch> bloch;
+  size_t next_local = 0, next_bloch = 0;
+  FxDensity density{};
+
+  static std::vector<double> transposed(const std::vector<double> &A, int m, int n) {
+    std::vector<double> t((size_t)m * n);
+    for (int i = 0; i < m; ++i)
+      for (int j = 0; j < n; ++j) t[(size_t)j * m + i] = A[(size_t)i * n + j];
+    return t;
+  }
+  explicit SfPlans(const paw_context *c)
+      : M(c->M1.data(), c->np1, c->np1),
+        D(c->D1.data(), c->np1, c->np1),
+        C(c->C1s.empty() ? c->M1.data() : c->C1s.data(), c->np1, c->np1, true),
+        phi(c->phiq.data(), c->nq1, c->np1),
+        pht(transposed(c->phiq, c->nq1, c->np1).data(), c->np1, c->nq1) {
+    const long double nP = phi.norm;
+    phi.put(density.phi, 1 / nP);
+    density.unit = (double)(nP * nP * nP);
+  }
+
+  // the entry to write next: a new one, or the oldest
+  template <class E>
+  static E &slot(std::vector<E> &v, size_t &next) {
+    if (v.size() < MAX) {
+      v.emplace_back();
+      return v.back();
+    }
+    E &e = v[next];
+    next = (next + 1) % MAX;
+    return e;
+  }
+
+  const FxBloch &bloch_tables(const paw_context *c, double alpha) {
+    for (const Bloch &e : bloch)
+      if (e.alpha == alpha) return e.t;
+    FxBloch t{};
+    const double f = alpha * (c->h / 2.0) * (c->h / 2.0);
+    const double kx = c->kvec[0], ky = c->kvec[1], kz = c->kvec[2];
+    // T: k_y C P + k_z M Q in the scale rho, then y = fC S + fM T in the scale 2^eta
+    const long double nM = M.norm, nC = C.norm, tiny = 1e-300;
+    const long double rho = std::max(((long double)std::fabs(ky) + std::fabs(kz)) * nC * nM, tiny);
+    const int eta = fx_scale((double)std::max(std::fabs(f) * (std::fabs(kx) * nC * nM * nM + nM * rho), tiny));
+    M.put(t.M, 1 / nM);
+    C.put(t.C, 1 / nC);
+    C.put(t.kyC, ky * nM / rho);
+    M.put(t.kzM, kz * nC / rho);
+    C.put(t.fC, std::ldexp(f * (kx * nM * nM), -eta));
+    M.put(t.fM, std::ldexp(f * rho, -eta));
+    t.eta = eta;
+    Bloch &e = slot(bloch, next_bloch);
+    e.alpha = alpha;
+    e.t = t;
+    return e.t;
+  }
+
+  const FxLocal &local_tables(const paw_context *c, double alpha_in, double cK, double cV, double cM) {
+    for (const Local &e : local)
+      if (e.alpha == alpha_in && e.cK == cK && e.cV == cV && e.cM == cM) return e.t;
+    FxLocal t{};
+    const double hh = c->h / 2.0, kf = cK * 0.5 * hh, mf = hh * hh * hh;
+    const long double tiny = 1e-300;
+    t.hasK = kf != 0.0;
+    t.doV = cV != 0.0;
+    t.bad = !std::isfinite(alpha_in) || !std::isfinite(kf) || !std::isfinite(cV);
+    const double alpha = t.bad ? 1.0 : alpha_in;
+    // scales (see FxLocal); without a kinetic part c is a power of two times cM
+    const long double nM = M.norm, nD = D.norm, nP = phi.norm, nT = pht.norm, p3 = nP * nP * nP, akf = std::fabs(kf);
+    const long double rho =
+        t.hasK ? akf * 2 * nD * nM * 16 / 15 : std::ldexp(mf * nM * nM, std::max(fx_scale(cM), -900));
+    t.room = t.hasK ? 4 : 1;
+    t.eta =
+        fx_scale((double)std::max(std::fabs(alpha) * (akf * nD * nM * nM + nM * rho) * (t.doV ? 4 : 3) / 3, tiny));
+    t.zeta = fx_scale((double)(std::ldexp((long double)0.5, t.eta) /
+                               std::max(std::fabs(alpha * cV) * p3 * nT * nT * nT, tiny))) - 1;
+    t.mf = (double)(mf * nM * nM / rho);
+    t.cM = cM;
+    const Local *near = nullptr;   // tables of another alpha: only the last stage differs
+    for (const Local &e : local)
+      if (e.cK == cK && e.cV == cV && e.cM == cM && !e.t.bad) near = &e;
+    if (near) {
+      t.phi = near->t.phi;
+      t.phit = near->t.phit;
+      t.M = near->t.M;
+      t.D = near->t.D;
+      t.kD = near->t.kD;
+      t.kM = near->t.kM;
+    } else {
+      phi.put(t.phi, 1 / nP);
+      pht.put(t.phit, 1 / nT);
+      M.put(t.M, 1 / nM);
+      D.put(t.D, 1 / nD);
+      D.put(t.kD, kf * nM / rho);
+      M.put(t.kM, kf * nD / rho);
+    }
+    D.put(t.fD, std::ldexp(alpha * (kf * nM * nM), -t.eta));
+    M.put(t.fM, std::ldexp(alpha * rho, -t.eta));
+    pht.put(t.fB, t.doV ? std::ldexp(alpha * (cV * p3 * nT * nT), t.zeta - t.eta) : 0);
+    Local &e = slot(local, next_local);
+    e.alpha = alpha_in;
+    e.cK = cK;
+    e.cV = cV;
+    e.cM = cM;
+    e.t = t;
+    return e.t;
+  }
+};
+
+static SfPlans &plans(paw_context *c) {
+  if (!c->sf_plans) c->sf_plans = std::make_shared<SfPlans>(c);
+  return *c->sf_plans;
+}
+
 void bloch_sf(paw_context *c, const double *X, int ldx, double *Y, int ldy, int ncols, double alpha,
               cudaStream_t s) {
   if (ncols <= 0 || !c->kc) return;
-  const int np1 = c->np1;
-  const Tab1 M(c->M1.data(), np1, np1), C(c->C1s.data(), np1, np1, true);
-  FxBloch t{};
-  const double f = alpha * (c->h / 2.0) * (c->h / 2.0);
-  const double kx = c->kvec[0], ky = c->kvec[1], kz = c->kvec[2];
-  // T: k_y C P + k_z M Q in the scale rho, then y = fC S + fM T in the scale 2^eta
-  const long double nM = M.norm, nC = C.norm, tiny = 1e-300;
-  const long double rho = std::max(((long double)std::fabs(ky) + std::fabs(kz)) * nC * nM, tiny);
-  const int eta = fx_scale((double)std::max(std::fabs(f) * (std::fabs(kx) * nC * nM * nM + nM * rho), tiny));
-  M.put(t.M, 1 / nM);
-  C.put(t.C, 1 / nC);
-  C.put(t.kyC, ky * nM / rho);
-  M.put(t.kzM, kz * nC / rho);
-  C.put(t.fC, std::ldexp(f * (kx * nM * nM), -eta));
-  M.put(t.fM, std::ldexp(f * rho, -eta));
+  FxBloch t = plans(c).bloch_tables(c, alpha);
   t.cell_dofs = c->cell_dofs.as<int>();
   t.X = X;
   t.Y = Y;
   t.ldx = ldx;
   t.ldy = ldy;
   t.ncols = ncols;
-  t.eta = eta;
   with_sizes(c, ncols, "degree out of range for the Bloch kernel",
              [&](auto np, auto vt) { launch_bloch<decltype(np)::value, decltype(vt)::value>(c, t, s); });
 }
@@ -751,11 +865,7 @@ void bloch_sf(paw_context *c, const double *X, int ldx, double *Y, int ldy, int 
 template <typename T>
 void density_sf(paw_context *c, const T *X, int ldx, int ncols, const double *wq, const double *f, double *out,
                 cudaStream_t s) {
-  const Tab1 phi(c->phiq.data(), c->nq1, c->np1);
-  FxDensity t{};
-  const long double nP = phi.norm;
-  phi.put(t.phi, 1 / nP);
-  t.unit = (double)(nP * nP * nP);
+  FxDensity t = plans(c).density;
   t.cell_dofs = c->cell_dofs.as<int>();
   t.wq = wq;
   t.f = f;
@@ -773,36 +883,7 @@ template void density_sf<float>(paw_context *, const float *, int, int, const do
 void local_sf(paw_context *c, const double *X, int ldx, double *Y, int ldy, int ncols, double alpha, double cK,
               double cV, double cM, const double *cMcol, cudaStream_t s) {
   if (ncols <= 0) return;
-  const int np1 = c->np1, nq1 = c->nq1;
-  std::vector<double> phit((size_t)np1 * nq1);
-  for (int q = 0; q < nq1; ++q)
-    for (int a = 0; a < np1; ++a) phit[(size_t)a * nq1 + q] = c->phiq[(size_t)q * np1 + a];
-  const Tab1 M(c->M1.data(), np1, np1), D(c->D1.data(), np1, np1);
-  const Tab1 phi(c->phiq.data(), nq1, np1), pht(phit.data(), np1, nq1);
-  FxLocal t{};
-  const double hh = c->h / 2.0, kf = cK * 0.5 * hh, mf = hh * hh * hh;
-  const long double tiny = 1e-300;
-  t.hasK = kf != 0.0;
-  t.doV = cV != 0.0;
-  t.bad = !std::isfinite(alpha) || !std::isfinite(kf) || !std::isfinite(cV);
-  if (t.bad) alpha = 1.0;
-  // scales (see FxLocal); without a kinetic part c is a power of two times cM
-  const long double nM = M.norm, nD = D.norm, nP = phi.norm, nT = pht.norm, p3 = nP * nP * nP, akf = std::fabs(kf);
-  const long double rho = t.hasK ? akf * 2 * nD * nM * 16 / 15 : std::ldexp(mf * nM * nM, std::max(fx_scale(cM), -900));
-  t.room = t.hasK ? 4 : 1;
-  t.eta = fx_scale((double)std::max(std::fabs(alpha) * (akf * nD * nM * nM + nM * rho) * (t.doV ? 4 : 3) / 3, tiny));
-  t.zeta = fx_scale((double)(std::ldexp((long double)0.5, t.eta) /
-                             std::max(std::fabs(alpha * cV) * p3 * nT * nT * nT, tiny))) - 1;
-  phi.put(t.phi, 1 / nP);
-  pht.put(t.phit, 1 / nT);
-  M.put(t.M, 1 / nM);
-  D.put(t.D, 1 / nD);
-  D.put(t.kD, kf * nM / rho);
-  M.put(t.kM, kf * nD / rho);
-  D.put(t.fD, std::ldexp(alpha * (kf * nM * nM), -t.eta));
-  M.put(t.fM, std::ldexp(alpha * rho, -t.eta));
-  pht.put(t.fB, t.doV ? std::ldexp(alpha * (cV * p3 * nT * nT), t.zeta - t.eta) : 0);
-  t.mf = (double)(mf * nM * nM / rho);
+  FxLocal t = plans(c).local_tables(c, alpha, cK, cV, cM);
   // w_q V_q per cell (rebuilt lazily after a potential change)
   if (!c->wV_valid) {
     c->wV.ensure(sizeof(fx2) * (size_t)c->ncells * c->nq, &c->dev_bytes);
@@ -818,7 +899,6 @@ void local_sf(paw_context *c, const double *X, int ldx, double *Y, int ldy, int 
   t.X = X;
   t.Y = Y;
   t.cMcol = cMcol;
-  t.cM = cM;
   t.ldx = ldx;
   t.ldy = ldy;
   t.ncols = ncols;
