@@ -149,11 +149,8 @@ __device__ __forceinline__ void fx_mac(long long &hh, long long &mm, int xh, int
   fx_mad(mm, xl, c.h);
 }
 
-// the sum of a pair of accumulators (mm started from FX_HALF), one IMAD.WIDE
-__device__ __forceinline__ long long fx_sum(long long hh, long long mm) {
-  fx_mad(hh, (int)(mm >> 32), 1);
-  return hh;
-}
+// the sum of a pair of accumulators (mm started from FX_HALF)
+__device__ __forceinline__ long long fx_sum(long long hh, long long mm) { return hh + (mm >> 32); }
 #endif
 
 }  // namespace pawfe

@@ -163,14 +163,14 @@ struct FxLocal {
   double cM, mf;        // c = (cM + cMcol[j]) mf, in the scale of S and R
   int64_t ldx, ldy;
   int ncols, ntile;
-  int hasK, doV, bad;   // bad: a factor is not finite
+  int hasK, hasM, doV, bad;   // bad: a factor is not finite
   int room, eta, zeta;   // room: |c| <= 2^-room of the range of R
 };
 
 // VT vectors per block, one line of a contraction per thread: the longest stage ((p+2)^2
 // lines) in one pass.  Eight vectors and two blocks per SM at degrees up to 6 (measured per
-// 256 vectors of 16^3 cells: 9.9 ms at degree 6 and 2.9 ms at degree 4, with four vectors and
-// three to five blocks 10.1 and 3.4 ms: fewer idle lanes in the stages of (p+1)^2 lines);
+// 256 vectors of 16^3 cells, before the sums of fx_sum left the IMAD pipe: 9.9 ms at degree 6 and
+// 2.9 ms at degree 4, with four vectors and three to five blocks 10.1 and 3.4 ms: fewer idle lanes in the stages of (p+1)^2 lines);
 // four for blocks of at most four vectors, and at degrees 7 and 8, whose lines need more
 // registers.
 constexpr int FX_VT = 8, FX_VT_SMALL = 4;
@@ -225,8 +225,9 @@ __device__ __forceinline__ int fx_gather(const int *cell_dofs, const T *X, int64
 }
 
 // What bounds it: the IMAD pipe, three IMAD.WIDE per product at 32 per clock and SM (measured;
-// 56.7k of 142k instructions per cell and vector at p = 6): 6.8 ms of the 9.9 ms per 256
-// vectors of 16^3 cells at p = 6, the rest barriers and dependent issue.  The same contractions
+// some 40% of all instructions at p = 6): 6.8 ms of the 9.5 ms per 256 vectors of 16^3 cells at
+// p = 6 (9.9 ms with the sums of the accumulator pairs on that pipe too), the rest barriers and
+// dependent issue.  The same contractions
 // with FP64 FMAs took 53.2 ms there (FP64 pipe 88% busy); p = 4: 2.9 ms.
 // The tables are kernel parameters, read by the IMADs as constant operands.  The nodal tensor
 // of the potential part grows in place to the (p+2)^3 Gauss points and back (W); the kinetic
@@ -296,10 +297,12 @@ __global__ void __launch_bounds__(fx_threads<NP, VT>(), fx_blocks<NP, VT>()) k_l
       P.mac(A.M, x);
       P.store(SX + o, NP * RN * VT);
     }
-    Acc<NP> Q;
-    Q.init();
-    Q.mac(A.D, x);
-    Q.store(SQ + o, NP * RN * VT);
+    if (A.hasK) {
+      Acc<NP> Q;
+      Q.init();
+      Q.mac(A.D, x);
+      Q.store(SQ + o, NP * RN * VT);
+    }
   }
   __syncthreads();
   // U3, Z = w V U3 and B2 = phi^T Z: lines along z of W, in registers
@@ -353,29 +356,29 @@ __global__ void __launch_bounds__(fx_threads<NP, VT>(), fx_blocks<NP, VT>()) k_l
     p.load(SX + o, RN * VT);
     Acc<NP> T;
     T.init();
-    T.mac(A.kD, p);
-    if (fx_fold<NP, NP>()) T.fold();
-    {
+    if (A.hasK) {
+      T.mac(A.kD, p);
+      if (fx_fold<NP, NP>()) T.fold();
       Halves<NP> q;
       q.load(SQ + o, RN * VT);
       T.mac(A.kM, q);
+      if (D > 0) T.fold(min(D, 63));
     }
-    if (D > 0) T.fold(min(D, 63));
     Acc<NP> S;
     S.init();
     S.mac(A.M, p);
+    S.store(SX + o, RN * VT);
+    if (A.hasM) {
 #pragma unroll
-    for (int i = 0; i < NP / 2; ++i) {
-      const long long a = S.E(i), b = S.O(i);
-      SX[o + i * RN * VT] = a + b;
-      SX[o + (NP - 1 - i) * RN * VT] = a - b;
-      fx_mac(T.eh[i], T.em[i], fx_hi(a), fx_lo(a), cm);
-      fx_mac(T.oh[i], T.om[i], fx_hi(b), fx_lo(b), cm);
-    }
-    if (NP & 1) {
-      const long long a = S.E(NP / 2);
-      SX[o + (NP / 2) * RN * VT] = a;
-      fx_mac(T.eh[NP / 2], T.em[NP / 2], fx_hi(a), fx_lo(a), cm);
+      for (int i = 0; i < (NP + 1) / 2; ++i) {
+        const long long a = S.E(i);
+        fx_mac(T.eh[i], T.em[i], fx_hi(a), fx_lo(a), cm);
+      }
+#pragma unroll
+      for (int i = 0; i < NP / 2; ++i) {
+        const long long b = S.O(i);
+        fx_mac(T.oh[i], T.om[i], fx_hi(b), fx_lo(b), cm);
+      }
     }
     T.store(SQ + o, RN * VT);
   }
@@ -396,12 +399,12 @@ __global__ void __launch_bounds__(fx_threads<NP, VT>(), fx_blocks<NP, VT>()) k_l
     const int D = sD[v];
     Acc<NP> y;
     y.init();
-    {
+    if (A.hasK) {
       Halves<NP> s;
       s.load(SX + ln * RN * VT + v, VT);
       y.mac(A.fD, s);
+      y.fold(min(D, 63));
     }
-    y.fold(min(max(D, 0), 63));
     {
       Halves<NP> r;
       r.load(SQ + ln * RN * VT + v, VT);
@@ -899,6 +902,7 @@ void local_sf(paw_context *c, const double *X, int ldx, double *Y, int ldy, int 
   t.X = X;
   t.Y = Y;
   t.cMcol = cMcol;
+  t.hasM = cMcol || t.cM != 0.0;
   t.ldx = ldx;
   t.ldy = ldy;
   t.ncols = ncols;
