@@ -29,7 +29,9 @@ constexpr int DG = 7;            // digits of an operand
 constexpr int DG_BITS = 54;      // |integer| < 2^54: the top digit stays within +-65
 constexpr int DG_SUMS = 8;       // accumulators: digit positions 5 .. 12
 constexpr int FLUSH = 9;         // k steps of 16 between two flushes
-constexpr int EXP_K = 128;       // coefficients of one batch of the expansion (8 k steps)
+// coefficients of one batch of the expansion: 8 k steps, or 7 where sums of several batches share
+// the shared memory (two blocks per SM at degree 6)
+constexpr int EXP_K = 128, EXP_K_MANY = 112;
 constexpr unsigned long long DG_BIAS = 0x80808080808080ull;
 
 // rows (nodes or coefficients) of VT FP16 digits; the 16-byte pieces of a row are placed so
@@ -152,6 +154,7 @@ __host__ __device__ __forceinline__ int sum_shift(int K) {
 
 struct FxNl {
   int n, p, N1, own, kt;          // kt: tiles of 16 owned nodes
+  int bp;                         // pairs of one batch of the expansion
   const int *own_off, *own_atom;
   const unsigned char *proj, *exp;   // digit images (operand A of the projection, of the expansion)
   const int *sP;                  // exponent per pair and projector: |P| < 2^sP
@@ -191,9 +194,9 @@ __device__ __forceinline__ void max_of_vectors(int (&E)[2], int *red, int *Em) {
 // pair is zero are skipped.
 // What bounds it: dependent issue of the digit steps (34 digit products per 16 x 8 x 16 tile keep
 // the tensor pipe 40% busy; the rest makes and flushes digits).  Projection and expansion of
-// 256 vectors of 16^3 cells of degree 6 with 64 atoms take 8.3 ms with the couplings, with FP64
+// 256 vectors of 16^3 cells of degree 6 with 64 atoms take 7.4 ms with the couplings, with FP64
 // FMAs on the nonzero entries 24.8 ms (FP64 pipe 80-95% busy).  Loading the next tile's bytes
-// ahead of the products was slower (9.5 against 9.2 ms: conversions done twice).
+// ahead of the products was slower (9.5 against 9.2 ms when the step was first made: conversions done twice).
 template <int NPAD, int VT, bool SCALED>
 __global__ void __launch_bounds__(256, 2) k_fx_project(FxNl A, const double *__restrict__ X, int64_t ldx, int ncols,
                                                        const double *__restrict__ rowscale, double *__restrict__ U) {
@@ -303,14 +306,18 @@ __global__ void __launch_bounds__(256, 2) k_fx_project(FxNl A, const double *__r
 
 // Expansion: one cell and VT vectors per block, a warp per (16 owned nodes, 16 vectors).  The
 // coefficients W of the cell's pairs, scaled by the pairs' projector exponents, are cut into
-// digits in batches of EXP_K; sums of several batches (more than EXP_K / NPAD pairs) and of the
-// first coefficient set of the recurrence wait in shared memory.
-// What bounds it: the mma rate, as in the projection.
+// digits in batches of bp pairs; sums of several batches wait in shared memory (digits
+// and sums of 32 vectors at degree 6 let two blocks share an SM).  The two coefficient sets of the
+// recurrence give one output each: T from W_S, then R_X from W_H.  (With the sums of W_S kept
+// beside those of W_H until one emission, one block fits an SM: a step of 128 vectors on 12^3
+// cells 13.7 instead of 8.0 ms.)
+// What bounds it: dependent issue of the digit steps, as in the projection.
 template <int NPAD, int VT, int MODE>
 __global__ void __launch_bounds__(256, 2) k_fx_expand(FxNl N, ExpArgs A, const double *__restrict__ W1,
                                                       const double *__restrict__ W2) {
-  constexpr int MT = NPAD / 16, H = VT / 16, VP = VT / 2, ROWS = 256 / VP, BP = EXP_K / NPAD;
-  constexpr int NW = (MODE == EXP_RECURRENCE) ? 2 : 1, plane = EXP_K * VT * 2, BIG = 1 << 20;
+  constexpr int MT = NPAD / 16, H = VT / 16, VP = VT / 2, ROWS = 256 / VP;
+  constexpr int NW = (MODE == EXP_RECURRENCE) ? 2 : 1, BIG = 1 << 20;
+  const int BP = N.bp, plane = BP * NPAD * VT * 2;
   extern __shared__ __align__(128) unsigned char sm[];
   __shared__ int red[8 * VT], Em[NW][VT], ooff[512];
   const int ncols = A.ncols, ntile = (ncols + VT - 1) / VT;
@@ -340,8 +347,8 @@ __global__ void __launch_bounds__(256, 2) k_fx_expand(FxNl N, ExpArgs A, const d
   }
   const unsigned smu = (unsigned)__cvta_generic_to_shared(sm);
   const int sh = sum_shift(max(np, 1) * NPAD), nbatch = max(1, (np + BP - 1) / BP);
-  const int units = N.kt * H, tot = N.kt * 16 * VT;
-  long long *S = reinterpret_cast<long long *>(sm + DG * plane);   // [NW][kt * 16][VT]
+  const int units = N.kt * H;
+  long long *S = reinterpret_cast<long long *>(sm + DG * plane);   // [kt * 16][VT]
   const int64_t base = owned_base(e, N.n, N.p, N.N1);
   for (int w = 0; w < NW; ++w) {
     const double *W = w ? W2 : W1;
@@ -350,8 +357,8 @@ __global__ void __launch_bounds__(256, 2) k_fx_expand(FxNl N, ExpArgs A, const d
       if (w || b) __syncthreads();
       for (int r = r0; r < pb * NPAD; r += ROWS) {
         double x, y;
-        get(W, b * EXP_K + r, x, y);
-        const int s = N.sP[(size_t)k0 * NPAD + b * EXP_K + r];
+        get(W, b * BP * NPAD + r, x, y);
+        const int s = N.sP[((size_t)k0 + b * BP) * NPAD + r];
         store_digits(sm, plane, piece<VT>(r, vp >> 2) + (vp & 3) * 4,
                      x == 0.0 ? 0 : fx_from<DG_BITS>(x, Em[w][2 * vp] - s),
                      y == 0.0 ? 0 : fx_from<DG_BITS>(y, Em[w][2 * vp + 1] - s));
@@ -375,7 +382,7 @@ __global__ void __launch_bounds__(256, 2) k_fx_expand(FxNl N, ExpArgs A, const d
             t.step<VT>(image<MT>(N.exp, kb + q, N.kt, kt, m), smu, plane, q * NPAD + m * 16, half);
         }
         t.flush(sh);
-        const bool last = b + 1 == nbatch && w + 1 == NW;
+        const bool last = b + 1 == nbatch;
         const int l0 = half * 16 + 2 * (lane & 3), e0 = 72 - sh - 2 * DG_BITS - 1022;
         auto value = [&](long long y, int E) {
           return E >= BIG ? __longlong_as_double(0x7ff8000000000000ll) : fx_to_small(y, e0 + E);
@@ -386,10 +393,10 @@ __global__ void __launch_bounds__(256, 2) k_fx_expand(FxNl N, ExpArgs A, const d
           long long *Sp = S + o * VT + l0;
           if (b > 0)
 #pragma unroll
-            for (int i = 0; i < 4; ++i) t.s[i >> 1][2 * r + (i & 1)] += Sp[w * tot + (i >> 1) * 8 + (i & 1)];
+            for (int i = 0; i < 4; ++i) t.s[i >> 1][2 * r + (i & 1)] += Sp[(i >> 1) * 8 + (i & 1)];
           if (!last) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) Sp[w * tot + (i >> 1) * 8 + (i & 1)] = t.s[i >> 1][2 * r + (i & 1)];
+            for (int i = 0; i < 4; ++i) Sp[(i >> 1) * 8 + (i & 1)] = t.s[i >> 1][2 * r + (i & 1)];
             continue;
           }
           if (o >= own) continue;
@@ -406,11 +413,11 @@ __global__ void __launch_bounds__(256, 2) k_fx_expand(FxNl N, ExpArgs A, const d
               Y[c] = value(s, Em[0][l0 + c]);
             } else if (MODE == EXP_SINV) {
               Y[c] = m * (Xi[c] - value(s, Em[0][l0 + c]));
+            } else if (w == 0) {
+              Y[c] = m * (Xi[c] - value(s, Em[0][l0 + c]));
             } else {
               double *RX = static_cast<double *>(A.RX) + d * A.ldx + v0 + l0 + c;
-              const double ry = Xi[c];
-              Y[c] = m * (ry - value(Sp[c], Em[0][l0 + c]));
-              const double bracket = -A.beta * ry - A.gamma * *RX + value(s, Em[NW - 1][l0 + c]);
+              const double bracket = -A.beta * Xi[c] - A.gamma * *RX + value(s, Em[NW - 1][l0 + c]);
               *RX = fma(A.c64[v0 + l0 + c], static_cast<const double *>(A.Y0)[d * A.ldy0 + v0 + l0 + c], bracket);
             }
           }
@@ -481,16 +488,21 @@ void launch_project(paw_context *c, const double *X, int ldx, int ncols, const d
   PAW_LAUNCH_CHECK("k_fx_project");
 }
 
-// shared memory of the expansion: the digits of a batch and, where sums have to wait, S
-size_t expand_smem(const paw_context *c, int mode, int vt) {
-  const int sets = (mode == EXP_RECURRENCE ? 1 : 0) + (c->max_own_pairs > EXP_K / c->npad ? 1 : 0);
-  return (size_t)vt * (DG * EXP_K * 2 + (size_t)sets * ((c->own + 15) / 16) * 16 * sizeof(long long));
+// shared memory of the expansion: the digits of a batch and, for cells of several, the sums
+int expand_pairs(const paw_context *c) {
+  return (c->max_own_pairs > EXP_K / c->npad ? EXP_K_MANY : EXP_K) / c->npad;
+}
+size_t expand_smem(const paw_context *c, int vt) {
+  const int bp = expand_pairs(c);
+  const size_t sums = c->max_own_pairs > bp ? ((c->own + 15) / 16) * 16 * sizeof(long long) : 0;
+  return (size_t)vt * (DG * bp * c->npad * 2 + sums);
 }
 
 template <int NPAD, int VT, int MODE>
 void launch_expand(paw_context *c, const ExpArgs &A, const double *W1, const double *W2, cudaStream_t s) {
-  const FxNl N = fx_args(c);
-  const size_t shm = expand_smem(c, MODE, VT);
+  FxNl N = fx_args(c);
+  N.bp = expand_pairs(c);
+  const size_t shm = expand_smem(c, VT);
   PAW_CUDA(cudaFuncSetAttribute(k_fx_expand<NPAD, VT, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
   k_fx_expand<NPAD, VT, MODE><<<(unsigned)((int64_t)c->ncells * ((A.ncols + VT - 1) / VT)), 256, shm, s>>>(N, A, W1,
                                                                                                          W2);
@@ -525,7 +537,7 @@ void nlfx_build(paw_context *c, const double *P) {
 
 // Blocks of 32 vectors share the digits and the projector images of a cell between two tiles of
 // 16; 16 vectors where there are no more, and where the rows of 32 vectors would not fit into
-// shared memory (degree 8; the recurrence at degree 7 with more than eight atoms on a cell).
+// shared memory (degree 8).
 constexpr size_t FX_SMEM_MAX = 200 * 1024;
 
 void nlfx_project(paw_context *c, const double *X, int ldx, int ncols, const double *rowscale, double *U,
@@ -544,7 +556,7 @@ void nlfx_project(paw_context *c, const double *X, int ldx, int ncols, const dou
 void nlfx_expand(paw_context *c, int mode, const ExpArgs &A, const double *W1, const double *W2, cudaStream_t s) {
   PAW_REQUIRE(c->max_own_pairs <= PAIRS_PER_CELL_MAX && c->own <= 512, PAW_ERR_UNSUPPORTED,
               "too many atoms on one cell for the expansion kernel");
-  const bool narrow = A.ncols <= 16 || expand_smem(c, mode, 32) > FX_SMEM_MAX;
+  const bool narrow = A.ncols <= 16 || expand_smem(c, 32) > FX_SMEM_MAX;
   if (c->npad == 16)
     narrow ? expand_mode<16, 16>(c, mode, A, W1, W2, s) : expand_mode<16, 32>(c, mode, A, W1, W2, s);
   else
