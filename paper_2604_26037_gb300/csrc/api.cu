@@ -374,6 +374,18 @@ static int cheb_cols(const paw_context *c, paw_precision prec, int nb) {
   const int64_t tiles = (int64_t)c->ncells * ((nb + 127) / 128);
   return (tc && !c->kc && c->tc_variant == 0 && tiles > 304) ? (nb + 3) / 4 * 4 : nb;
 }
+// Early starts (launch_pdl) for the loop of a small block: 16 vectors on 4^3 cells of degree 4, 20
+// steps: 595 instead of 752 us; 256 vectors in blocks of 32 on 8^3 cells of degree 5: 20.8 instead
+// of 22.3 ms.  With many tiles per SM the waiting blocks of the next kernel cost more than their
+// start-up (12^3 cells of degree 5, blocks of 128: 27.3 against 26.7 ms), and in a batch they would
+// hold SMs that other instances could use.
+struct PdlIssue {
+  paw_context *c;
+  PdlIssue(paw_context *ctx, int ncols) : c(ctx) {
+    c->pdl = (int64_t)c->ncells * ((ncols + 127) / 128) <= 608 ? 1 : 0;
+  }
+  ~PdlIssue() { c->pdl = 0; }
+};
 struct PaddedIssue {
   paw_context *c;
   PaddedIssue(paw_context *ctx, int mode) : c(ctx) { c->padded = mode; }
@@ -402,6 +414,7 @@ static void block_step2(paw_context *c, const double *X, int ldx, int nb, int nb
 template <typename TR>
 static void block_loop(paw_context *c, paw_precision prec, const double *X, int ldx, int nout, int nb, double a0,
                        double cc, const ChebScalars &S, int par, double *Xo, int ldo, cudaStream_t s) {
+  c->u_clean = 0;
   const PaddedIssue padded(c, nb != nout ? PAD_SAME : PAD_NONE);   // nb columns are worked on, nout belong to the block
   const int64_t M = c->ndof;
   const int nsteps = S.nsteps;
@@ -486,6 +499,7 @@ static void block_loop(paw_context *c, paw_precision prec, const double *X, int 
   {
     PhaseScope ps(c, 5, s);
     op_Sinv<TR>(c, prec, RY, ldr, T, ldr, nb, s);
+    c->u_clean = 0;
     k_cheb_recover<TR><<<ew_grid(M, nout), blk, 0, s>>>(M, nout, T, ldr, X, ldx, d_lyfin, Xo, ldo);
     PAW_LAUNCH_CHECK("k_cheb_recover");
   }
@@ -552,6 +566,7 @@ static void cheb_block(paw_context *c, paw_precision prec, const double *X, int 
   cheb_plan(nbp, m, bd, lamp.data(), S, hd, hf);
   const double *hd_dev = static_cast<const double *>(sl.dev);
   try {
+    const PdlIssue pdl(c, nb);
     cheb_issue(c, prec, X, ldx, nb, nbp, bd, S, hd, hf, Xo, ldo, s, hd_dev, reinterpret_cast<const float *>(hd_dev + nd));
   } catch (...) {
     // copies from the slot may already be enqueued: keep it until the stream passes them
@@ -569,7 +584,7 @@ static void cheb_block(paw_context *c, paw_precision prec, const double *X, int 
 // their SMs, so step 2 advances where they leave SMs idle (at their ends and in small problems):
 // 1-7% per call.  (Forms of the loop kernels with half the shared memory, beside which blocks of
 // step 2 fit, were 24% slower and hid an FP64-pipe-bound step 2 of 78 ms per 256 vectors; beside
-// the present one of 18 ms the mid call takes 190.5 ms with them and 186.1 ms without.)  Blocks
+// one of 18 ms the mid call takes 190.5 ms with them and 186.1 ms without.)  Blocks
 // of parity j & 1 use the parity's Y buffer and scalar images; the side stream reuses them for
 // block j + 2 only after the loop of block j has finished.
 static cudaEvent_t next_event(paw_context *c) {
@@ -650,6 +665,7 @@ static void cheb_filter_overlapped(paw_context *c, paw_precision prec, const dou
     if (j + 1 < nbk) issue_step2(j + 1);
     const int j0 = j * B, nb = std::min(B, ncols - j0), nr = cw * nb;
     PAW_CUDA(cudaStreamWaitEvent(c->s_loop, evY[j], 0));
+    const PdlIssue pdl(c, nr);
     if (c->kc) {
       double *Y = c->ws_cyp[j & 1].as<double>();
       block_loop<float>(c, prec, block_in(j), nr, nr, nr, bd.a0, cc, S[j], j & 1, Y, nr, c->s_loop);

@@ -384,14 +384,15 @@ static void cell_stream(paw_context *c, const TcMats &T, const float *X, int ldx
   p.alpha = alpha;
   encode_row_map(&p.tm, X, c->ndof, ncols, ldx);
   const size_t shm = tcs::Geo<P>::SMEM;
-  PAW_CUDA(cudaFuncSetAttribute(tcs::k_tc_stream<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+  auto kern = c->pdl ? tcs::k_tc_stream<P, true> : tcs::k_tc_stream<P, false>;
+  PAW_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
   int dev = 0, nsm = 0;
   PAW_CUDA(cudaGetDevice(&dev));
   PAW_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
   const int cap = c->grid_cap > 0 ? std::min(c->grid_cap, nsm) : nsm;
   const int grid = std::max(1, std::min(p.ntiles, cap));
-  tcs::k_tc_stream<P><<<grid, tcs::threads_for(P::NEPI), shm, s>>>(p, c->status_dev.as<int>(), c->wait_ns,
-                                                                     c->wait_probe);
+  launch_pdl(c, kern, grid, tcs::threads_for(P::NEPI), shm, s, p, c->status_dev.as<int>(), c->wait_ns,
+             c->wait_probe);
   PAW_LAUNCH_CHECK("k_tc_stream<cell>");
 }
 

@@ -238,6 +238,8 @@ struct paw_context {
   // and the scalar images of the block (FP64 -Lambda, Lambda_Y, alpha Lambda_Y;
   // FP32 hi/lo words)
   pawfe::DevBuf ws_Y0p[2], ws_lamp[2], ws_cfp[2];
+  int pdl = 0;       // 1: launch_pdl may let a kernel start before the one before it has ended
+  int u_clean = 0;   // 1: the projection sums U were zeroed by the last expansion of the loop
   int padded = 0;    // PAD_*: work on a block padded to whole 16-byte rows is being issued
   cudaStream_t s_loop = nullptr, s_side = nullptr;   // internal streams of the overlapped filter
   std::vector<cudaEvent_t> ev_pool;
@@ -264,6 +266,25 @@ struct paw_context {
 };
 
 namespace pawfe {
+
+// ---------------------------------------------------------------- launches
+// Launch of a kernel that begins with grid_wait() (tc_ptx.cuh): while c->pdl is set, its start-up
+// (launch latency, barriers, tensor memory) overlaps the end of the kernel before it on the
+// stream.  The kernels of the filter's loop in the tensor-core forms are launched this way.
+template <class... P, class... A>
+void launch_pdl(const paw_context *c, void (*kernel)(P...), dim3 grid, dim3 block, size_t shm, cudaStream_t s, const A &...args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = shm;
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = c->pdl;
+  PAW_CUDA(cudaLaunchKernelEx(&cfg, kernel, args...));
+}
 
 // ---------------------------------------------------------------- setup.cu
 void build_tables(paw_context *c);

@@ -23,6 +23,7 @@
 
 #include "common.cuh"
 #include "nonlocal_common.cuh"
+#include "tc_ptx.cuh"
 
 namespace pawfe {
 
@@ -300,12 +301,15 @@ __global__ void __launch_bounds__(NPAD * NPAD) k_couple_f(int npj, const int *__
 // slots s = goff[a] + w, + NW, ... into all npj rows, the NW partial sums meet in
 // shared memory.  F rows are warp-uniform float4 loads (padded columns are zero),
 // U columns coalesced 128-byte loads.  Rows al >= npj of W_S and W_H are zero.
+// (U, written by the kernel before, is read with plain loads: the launch may begin before that
+// kernel has ended.)
 template <int NPAD, int NW>
 __global__ void __launch_bounds__(NW * 32) k_own_couple_sh(int npj, const int *__restrict__ goff,
                                                            const int *__restrict__ gatom, const float *__restrict__ F,
-                                                           const float *__restrict__ Ds, const float *__restrict__ U,
-                                                           float alpha, float *__restrict__ WS,
-                                                           float *__restrict__ WH, int ncols) {
+                                                           const float *__restrict__ Ds, const float *U, float alpha,
+                                                           float *WS, float *WH, int ncols) {
+  tcp::grid_wait();
+  tcp::grid_dependents();
   __shared__ float red[NW][NPAD][32];
   const int a = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int v = blockIdx.y * 32 + lane;
@@ -699,6 +703,7 @@ static T *project_U(paw_context *c, paw_precision prec, const T *X, int ldx, int
   if constexpr (sizeof(T) == 4) {
     if (use_tc<T>(c, prec)) {
       if (nltc_project(c, X, ldx, ncols, rowscale, PP, U, s)) return U;   // reduced in the epilogue
+      c->u_clean = 0;
       dim3 g((ncols + 31) / 32, c->npad, c->natoms);
       k_pair_reduce<T><<<g, 32, 0, s>>>(c->apair_off.as<int>(), c->apair.as<int>(), PP, c->npad, ncols, U);
       PAW_LAUNCH_CHECK("k_pair_reduce");
@@ -786,11 +791,11 @@ void nl_project_filter(paw_context *c, paw_precision prec, const T *RY, int ldr,
       dim3 g(c->natoms, (ncols + 31) / 32);
       const int *go = c->gnb_off.as<int>(), *ga = c->gnb_atom.as<int>();
       if (c->npad == 16)
-        k_own_couple_sh<16, 8><<<g, 8 * 32, 0, s>>>(c->npj, go, ga, c->Fsh32.as<float>(), c->DSinv32.as<float>(), U,
-                                                    (float)alpha, WS, WH, ncols);
+        launch_pdl(c, k_own_couple_sh<16, 8>, g, 8 * 32, 0, s, c->npj, go, ga, c->Fsh32.as<float>(),
+                   c->DSinv32.as<float>(), U, (float)alpha, WS, WH, ncols);
       else
-        k_own_couple_sh<32, 4><<<g, 4 * 32, 0, s>>>(c->npj, go, ga, c->Fsh32.as<float>(), c->DSinv32.as<float>(), U,
-                                                    (float)alpha, WS, WH, ncols);
+        launch_pdl(c, k_own_couple_sh<32, 4>, g, 4 * 32, 0, s, c->npj, go, ga, c->Fsh32.as<float>(),
+                   c->DSinv32.as<float>(), U, (float)alpha, WS, WH, ncols);
       PAW_LAUNCH_CHECK("k_own_couple_sh");
       return;
     }

@@ -596,6 +596,8 @@ struct Args {
   const float *W1, *W2;
   const float *mdo;   // M_D^-1 in owner order, nh * ntile per cell
   const int *odof;    // DoF indices in owner order, same layout
+  float *zero;        // cleared by the launch (nzero entries)
+  int64_t nzero;
 };
 
 struct Tile {
@@ -619,7 +621,12 @@ __device__ __forceinline__ Tile tile_of(const Args &a, int t) {
   return T;
 }
 
-template <int MODE>
+template <bool EARLY>
+__device__ __forceinline__ float load_w(const float *p) { return EARLY ? __ldca(p) : __ldg(p); }
+
+// EARLY: launched before the kernel before it has ended (launch_pdl); W, which that kernel writes,
+// is then read with coherent loads.
+template <int MODE, bool EARLY>
 __global__ void __launch_bounds__(THREADS, 1) k_exp_stream(const __grid_constant__ Args a, int *status) {
   using G = Geo<MODE>;
   constexpr int S = G::S;
@@ -644,7 +651,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_exp_stream(const __grid_constant
       mbar_init(smem_u32(&sh->sempty[b]), NEPI);
     }
     mbar_init(smem_u32(&sh->drain), 1);
-    sh->abort = (*reinterpret_cast<volatile int *>(status) != 0) ? 1 : 0;
+    if constexpr (!EARLY) sh->abort = (*reinterpret_cast<volatile int *>(status) != 0) ? 1 : 0;
     fence_barrier_init();
     fence_proxy_async();
   }
@@ -653,9 +660,14 @@ __global__ void __launch_bounds__(THREADS, 1) k_exp_stream(const __grid_constant
     tmem_alloc(smem_u32(&sh->taddr), 512);
     tmem_relinquish();
   }
+  if constexpr (EARLY) {
+    grid_wait();
+    if (threadIdx.x == 0) sh->abort = (*reinterpret_cast<volatile int *>(status) != 0) ? 1 : 0;
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  if constexpr (EARLY) grid_dependents();
   const uint32_t tmem = sh->taddr;
   volatile int *abort = &sh->abort;
   const uint32_t bbytes = (uint32_t)a.ntile * 128u;
@@ -748,8 +760,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_exp_stream(const __grid_constant
           const size_t rowb = ((size_t)(live ? a.A.own_atom[T.k0 + kk] : 0) * a.npad + al0) * ncols + v;
 #pragma unroll
           for (int i = 0; i < 16; ++i) {
-            f[0][hh * 16 + i] = live ? __ldg(a.W1 + rowb + (size_t)i * ncols) : 0.f;
-            if constexpr (G::NW == 2) f[G::NW - 1][hh * 16 + i] = live ? __ldg(a.W2 + rowb + (size_t)i * ncols) : 0.f;
+            f[0][hh * 16 + i] = live ? load_w<EARLY>(a.W1 + rowb + (size_t)i * ncols) : 0.f;
+            if constexpr (G::NW == 2) f[G::NW - 1][hh * 16 + i] = live ? load_w<EARLY>(a.W2 + rowb + (size_t)i * ncols) : 0.f;
           }
         }
         if (g >= (uint32_t)S && !tcs::wait_or_abort(smem_u32(&sh->empty[s]), (u - 1) & 1u, abort)) {
@@ -812,7 +824,10 @@ __global__ void __launch_bounds__(THREADS, 1) k_exp_stream(const __grid_constant
       }
     __syncwarp();
   } else if (warp < WARP_E0) {
-    // idle
+    // the sums of the next projection, read by the couplings before this launch, start from zero
+    // (a memset between the kernels would end the chain of early starts)
+    if constexpr (EARLY)
+      for (int64_t i = (int64_t)blockIdx.x * 32 + lane; i < a.nzero; i += (int64_t)gridDim.x * 32) a.zero[i] = 0.f;
   } else {
     // ---------------------------------------------------------------- epilogue
     const int q = warp & 3, part = (warp - WARP_E0) >> 2;
@@ -1008,10 +1023,11 @@ static int persistent_grid(const paw_context *c) {
 template <class P>
 static void launch_stream(const paw_context *c, const P &p, cudaStream_t s, const char *what) {
   const size_t shm = tcs::Geo<P>::SMEM;
-  PAW_CUDA(cudaFuncSetAttribute(tcs::k_tc_stream<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+  auto kern = c->pdl ? tcs::k_tc_stream<P, true> : tcs::k_tc_stream<P, false>;
+  PAW_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
   const int grid = std::max(1, std::min(p.ntiles, persistent_grid(c)));
-  tcs::k_tc_stream<P><<<grid, tcs::threads_for(P::NEPI), shm, s>>>(p, c->status_dev.as<int>(), c->wait_ns,
-                                                                     c->wait_probe);
+  launch_pdl(c, kern, grid, tcs::threads_for(P::NEPI), shm, s, p, c->status_dev.as<int>(), c->wait_ns,
+             c->wait_probe);
   PAW_LAUNCH_CHECK(what);
 }
 
@@ -1042,7 +1058,8 @@ static void proj_stream(paw_context *c, const float *X, int ldx, int ncols, bool
   p.U = U;
   p.mdo = N.mdo.as<float>();
   p.ostride = N.nh * N.ntile;
-  PAW_CUDA(cudaMemsetAsync(U, 0, sizeof(float) * (size_t)c->natoms * c->npad * ncols, s));
+  if (!c->u_clean) PAW_CUDA(cudaMemsetAsync(U, 0, sizeof(float) * (size_t)c->natoms * c->npad * ncols, s));
+  c->u_clean = 0;
   encode_row_map(&p.tm, X, c->ndof, ncols, ldx);
   launch_stream(c, p, s, "k_tc_stream<projection>");
 }
@@ -1125,9 +1142,17 @@ static void expand_stream(paw_context *c, const ExpArgs &A, const float *W1, con
       p.amask |= 1 << k;
     }
   const size_t shm = xs::smem_bytes<MODE>();
-  PAW_CUDA(cudaFuncSetAttribute(xs::k_exp_stream<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+  auto kern = c->pdl ? xs::k_exp_stream<MODE, true> : xs::k_exp_stream<MODE, false>;
+  PAW_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
   const int grid = std::max(1, std::min(p.ntiles, persistent_grid(c)));
-  xs::k_exp_stream<MODE><<<grid, xs::THREADS, shm, s>>>(p, c->status_dev.as<int>());
+  p.zero = nullptr;
+  p.nzero = 0;
+  if (MODE == EXP_RECURRENCE && !c->kc && c->pdl) {   // the next step projects into the same sums
+    p.zero = c->scr->partial.as<float>();
+    p.nzero = (int64_t)c->natoms * c->npad * A.ncols;
+    c->u_clean = 1;
+  }
+  launch_pdl(c, kern, grid, xs::THREADS, shm, s, p, c->status_dev.as<int>());
   PAW_LAUNCH_CHECK("k_exp_stream");
 }
 

@@ -66,6 +66,13 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t
 // consecutive box-sized rows of shared memory at dst (TMA tile::gather4; the
 // map's box is one row high); completes on mbarrier bar.  x * element size
 // must be a multiple of 16 bytes.
+// Programmatic dependent launch: a kernel launched with launch_pdl may start while the kernel
+// before it on the stream is still running, once every block of that one has called
+// grid_dependents() or ended; until grid_wait() returns (the kernel before has ended and its
+// writes are visible) it touches nothing that an earlier kernel writes.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 __device__ __forceinline__ void tma_gather4(uint32_t dst, const void *map, int x, int row0, int row1, int row2,
                                             int row3, uint32_t bar) {
   asm volatile(
