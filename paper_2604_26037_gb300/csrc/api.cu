@@ -931,17 +931,21 @@ static void apply_any(paw_context *c, paw_precision prec, int which, const void 
     // rows that are not whole 16-byte pieces: through zero-padded copies, on which the persistent
     // tensor-core kernels run (approximate inverse overlap, degree 6, 12^3 cells, 130 columns: 0.67
     // instead of 1.03 ms; H 1.14 instead of 1.69 ms; no slower on 4^3 cells of degree 4)
-    const int np = (ncols + 3) / 4 * 4;
+    // in blocks of at most 512 columns, which bounds the copies
+    const int np = std::min((ncols + 3) / 4 * 4, 512);
     c->ws_cx.ensure(sizeof(float) * (size_t)c->ndof * np, &c->dev_bytes);
     c->ws_cy.ensure(sizeof(float) * (size_t)c->ndof * np, &c->dev_bytes);
     float *xs = c->ws_cx.as<float>(), *ys = c->ws_cy.as<float>();
     const PaddedIssue padded(c, PAD_CELL);
-    copy_rows((const float *)X, ldx, ncols, xs, np, np, c->ndof, s);
-    if (which == 0)
-      op_H<float>(c, prec, xs, np, ys, np, np, s);
-    else
-      op_Sinv<float>(c, prec, xs, np, ys, np, np, s);
-    copy_rows(ys, np, ncols, (float *)Y, ldy, ncols, c->ndof, s);
+    for (int j = 0; j < ncols; j += np) {
+      const int n = std::min(np, ncols - j), m = (n + 3) / 4 * 4;
+      copy_rows((const float *)X + j, ldx, n, xs, m, m, c->ndof, s);
+      if (which == 0)
+        op_H<float>(c, prec, xs, m, ys, m, m, s);
+      else
+        op_Sinv<float>(c, prec, xs, m, ys, m, m, s);
+      copy_rows(ys, m, n, (float *)Y + j, ldy, n, c->ndof, s);
+    }
     return;
   }
   if (prec == PAW_FP64) {

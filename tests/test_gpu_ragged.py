@@ -47,7 +47,7 @@ def test_filter_blocks(prec, tol, ncols):
     assert (got[:, 0] == 9.0).all() and (got[:, 1 + ncols:] == 9.0).all()
 
 
-@pytest.mark.parametrize("ncols,off,extra", [(1, 0, 0), (6, 0, 0), (8, 1, 0), (8, 0, 1), (130, 3, 2)])
+@pytest.mark.parametrize("ncols,off,extra", [(1, 0, 0), (6, 0, 0), (8, 1, 0), (8, 0, 1), (130, 3, 2), (517, 1, 0)])
 def test_operators(ncols, off, extra):
     """Column counts, offsets and pitches that four does not divide, inside wider arrays."""
     import torch
