@@ -419,7 +419,7 @@ def run_ours(args, ws, rank, local):
         fp64 = {"value": whole_job_rate(units_per_step, ws, ms64), "ms_per_step": ms64,
                 "steps": args.fp64_steps, "warmup": 1}
 
-    # the same filter with step 2 in pair-of-FP32 arithmetic (FP64-class accuracy on the FP32 pipes)
+    # the same filter with options.y0_pair32 (served by the FP64 kernels of step 2)
     pair = None
     if args.pair_steps > 0 and not kp and not args.y0_pair32:
         fe_p = P.PawFE.from_system(sysd, block=cfg["block"], y0_fp32=args.y0_fp32, y0_pair32=True,
@@ -439,8 +439,7 @@ def run_ours(args, ws, rank, local):
                 "steps": args.pair_steps, "warmup": 1, "phases_ms_per_step": ph,
                 "step2_ms": round(s2, 3), "step2_speedup_vs_fp64": round(s2_64 / s2, 3),
                 "fp64_bracket_output_rel_diff": diff64, "clocks": clk_p,
-                "arithmetic": "step 2 with every product and sum on pairs of FP32 numbers (about 48 bits); "
-                              "Y stored FP64; the rest of the call as the main measurement"}
+                "arithmetic": "options.y0_pair32: step 2 by the same FP64-accurate kernels as without it"}
         del out_p
         fe_p.close()
 
@@ -598,7 +597,10 @@ def run_ours(args, ws, rank, local):
     # roofline of the dominant phase
     peaks = _peaks()
     phases = {k: v for k, v in prof.items() if isinstance(v, dict)}
-    dom = max(phases, key=lambda k: phases[k]["ms"])
+    # (by each phase's own time where the blocks were also run one after another: an interval of the
+    # overlapped schedule includes the time in which the other stream's kernels hold the SMs)
+    own = phases if iso_run is None else {k: v for k, v in iso_run[1].items() if isinstance(v, dict)}
+    dom = max(own, key=lambda k: own[k]["ms"])
     roof = roofline(dom, phases[dom], fe, sysd, cfg, args.prec, peaks, clocks, args.workload)
     all_roof = {k: roofline(k, v, fe, sysd, cfg, args.prec, peaks, clocks, args.workload) for k, v in phases.items()}
     # each kernel's own rate (blocks one after another), beside the timed region's
@@ -611,8 +613,6 @@ def run_ours(args, ws, rank, local):
                f"calls after the timed region: {ms_s:.1f} ms per call")
         roof["isolated"] = {kk: iso[dom][kk] for kk in ("achieved", "frac", "ms_per_launch") if kk in iso[dom]}
         roof["isolated"]["source"] = src
-        if "peak_alt" in iso[dom]:
-            roof["isolated"]["frac_alt"] = iso[dom]["peak_alt"]["frac"]
         roof["schedule"] = ("timed region: step 2 of block 0 alone, step 2 of block 1 beside the loop of block 0, "
                             "so the average launch duration includes the SMs shared with the loop")
         for k in all_roof:
@@ -633,7 +633,7 @@ def run_ours(args, ws, rank, local):
         "data": "synthetic (seeded), inputs resident in HBM and larger than L2",
         "config": {"workload": workload_desc(args.workload),
                    "precision": args.prec, "y0_storage": "fp32" if args.y0_fp32 else "fp64",
-                   "step2_arithmetic": "pair-of-FP32" if args.y0_pair32 else "fp64",
+                   "step2_arithmetic": "fp64",
                    **({"kpoint_per_bohr": list(kp), "vectors": "complex (real blocks of 2 B columns inside)"}
                       if kp else {}),
                    "start": args.start,
@@ -671,8 +671,8 @@ def fe_np1(nc):
 
 # kernels that make up each profiled phase of the filter (library phase brackets)
 PHASE_KERNELS = {
-    "residual_local": "k_local_sf (FP64 even/odd sum-factorised 1/2 K + V - lambda M)",
-    "residual_nonlocal": "k_own_project64 + k_pair_reduce + k_own_couple + k_own_expand64 (FP64)",
+    "residual_local": "k_local_fx (even/odd sum-factorised 1/2 K + V - lambda M, 64-bit fixed point)",
+    "residual_nonlocal": "k_fx_project + k_pair_reduce + k_own_couple + k_fx_expand (FP64 as FP16 digit products)",
     "recurrence": "k_exp_stream (tcgen05: fused Shat^-1 expansion + nonlocal H + recurrence update)",
     "projection": "k_tc_stream<ProjStream> + k_own_couple_sh (W_S and W_H from U)",
     "cell_products": "k_tc_stream<CellStream> (tcgen05 TF32/BF16) or k_cell_simt",
@@ -688,8 +688,8 @@ MEASURED_TRAFFIC = {
     ("cell_products", "tf32"): (23.17, "k_tc_stream<CellStream>", "mid"),
     ("recurrence", "tf32"): (25.60, "k_exp_stream<2>", "mid"),
     ("projection", "tf32"): (5.584, "k_tc_stream<ProjStream>", "mid"),
-    ("residual_local", None): (30.88, "k_local_sf<7,double>", "prof12"),
-    ("residual_nonlocal", None): (32.33, "k_own_project64<16,double> + k_own_expand64<16,0,double>", "prof12"),
+    ("residual_local", None): (24.1, "k_local_fx<7,8>", "prof12"),
+    ("residual_nonlocal", None): (25.0, "k_fx_project<16,32,0> + k_fx_expand<16,32,0>", "prof12"),
 }
 
 
@@ -705,7 +705,7 @@ def measured_traffic(phase, prec, units, workload):
 
 
 def sf_flops_per_cell_vec(n1):
-    """FP64 flops of the even/odd sum-factorised (1/2 K + V - lambda M) x per cell and vector
+    """Flops of the even/odd sum-factorised (1/2 K + V - lambda M) x per cell and vector
     (n1 nodes and n1 + 1 Gauss points per direction; FMA = 2 flops, add or multiply = 1)."""
     q1 = n1 + 1
 
@@ -749,22 +749,22 @@ def phase_model(phase, fe, cfg, prec):
     es = 4 if f32 else 8
     if phase == "cell_products":
         mat_es = {"bf16": 2, "tf32": 4, "fp32": 4, "fp64": 8}[prec]
-        if prec == "fp64":   # sum-factorised local H in FP64
-            return float(sf_flops_per_cell_vec(n1)) * ncells * B, M * B * 8 * 3, "fp64"
+        if prec == "fp64":   # sum-factorised local H
+            return float(sf_flops_per_cell_vec(n1)) * ncells * B, M * B * 8 * 3, "fixed64"
         kind = {"tf32": "tf32", "bf16": "bf16", "fp32": "fp32"}[prec]
         return 2.0 * ncells * nc * nc * B, ncells * nc * nc * mat_es + M * B * 4 * 3, kind
     if phase == "residual_local":
-        return float(sf_flops_per_cell_vec(n1)) * ncells * B, M * B * 8 * 3, "fp64"
+        return float(sf_flops_per_cell_vec(n1)) * ncells * B, M * B * 8 * 3, "fixed64"
     pbytes = nnz * es
     if phase == "projection":
-        return (2.0 * nnz * B, M * B * es + pbytes + 2 * pairs * fe.nproj * B * es, "fp32" if f32 else "fp64")
+        return (2.0 * nnz * B, M * B * es + pbytes + 2 * pairs * fe.nproj * B * es, "fp32" if f32 else "digit64")
     if phase == "recurrence":
         # reads R_Y, R_X and Y (an FP32 hi/lo pair or FP64: 8 bytes), writes T and R_X
-        return (4.0 * nnz * B, M * B * (es * 4 + 8) + pbytes, "fp32" if f32 else "fp64")
+        return (4.0 * nnz * B, M * B * (es * 4 + 8) + pbytes, "fp32" if f32 else "digit64")
     if phase == "residual_nonlocal":
-        return (4.0 * nnz * B, M * B * 8 * 3 + 2 * nnz * 8, "fp64")
+        return (4.0 * nnz * B, M * B * 8 * 3 + 2 * nnz * 8, "digit64")
     if phase == "recovery":
-        return (4.0 * nnz * B, M * B * (es * 2 + 8 * 2), "fp32" if f32 else "fp64")
+        return (4.0 * nnz * B, M * B * (es * 2 + 8 * 2), "fp32" if f32 else "digit64")
     return None, None, None
 
 
@@ -778,10 +778,18 @@ def compute_peak(kind, peaks, sm_mhz):
                 f"{peaks['src']} BF16 burst {peaks['bf16']} TFLOP/s x nominal TF32/BF16 ratio 1.1/2.25")
     if kind == "bf16":
         return peaks["bf16"], "tensor", f"{peaks['src']} BF16 burst"
-    if kind == "fp64":
-        # the FP64 pipe retires 2 FMA per SM per clock on GB300 (1.25 TFLOP/s nominal at 2070 MHz)
-        return (nsm * 2 * 2 * sm_mhz * 1e6 / 1e12, "alu",
-                f"derived: {nsm} SMs x 2 FP64 FMA/clk x 2 flop x {sm_mhz:.0f} MHz (median sampled SM clock)")
+    if kind == "fixed64":
+        # a 64-bit fixed-point product is three IMAD.WIDE, of which an SM retires 32 per clock
+        # (measured); the FP64 unit, 2 FMA per SM per clock, is not used
+        return (nsm * 32 / 3 * 2 * sm_mhz * 1e6 / 1e12, "alu",
+                f"derived: {nsm} SMs x 32 IMAD.WIDE/clk / 3 per product x 2 flop x {sm_mhz:.0f} MHz "
+                "(median sampled SM clock)")
+    if kind == "digit64":
+        # a product of two numbers of seven FP16 digits is 34 digit products; mma.sync retires
+        # 1024 of them per SM per clock (measured)
+        return (nsm * 1024 / 34 * 2 * sm_mhz * 1e6 / 1e12, "tensor",
+                f"derived: {nsm} SMs x 1024 FP16 mma.sync products/clk / 34 digit products x 2 flop x "
+                f"{sm_mhz:.0f} MHz (median sampled SM clock)")
     return (nsm * 128 * 2 * sm_mhz * 1e6 / 1e12, "alu",
             f"derived: {nsm} SMs x 128 FP32 lanes x 2 flop x {sm_mhz:.0f} MHz (median sampled SM clock)")
 
@@ -806,16 +814,9 @@ def roofline(phase, pinfo, fe, sysd, cfg, prec, peaks, clocks, workload=None):
               "ms_per_launch": round(per_launch_ms, 4), "algorithmic_bytes_per_launch": byts,
               "algorithmic_flops_per_launch": flops}
     if c_frac >= hbm_frac:
-        out = {"bound": cbound, "achieved": round(tfs, 3), "peak": round(cpk, 4), "unit": "TFLOP/s",
-               "frac": round(c_frac, 4), "hbm_frac": round(hbm_frac, 4), "compute": kind, "peak_source": csrc,
-               **common}
-        if kind == "fp64":
-            # the same kernel against the other admissible ceiling: the measured BF16 burst x the
-            # nominal FP64/BF16 ratio (1.25 / 2250)
-            alt = peaks["bf16"] * 1.25 / 2250.0
-            out["peak_alt"] = {"peak": round(alt, 4), "frac": round(tfs / alt, 4),
-                               "source": f"{peaks['src']} BF16 burst x nominal FP64/BF16 ratio 1.25/2250"}
-        return out
+        return {"bound": cbound, "achieved": round(tfs, 3), "peak": round(cpk, 4), "unit": "TFLOP/s",
+                "frac": round(c_frac, 4), "hbm_frac": round(hbm_frac, 4), "compute": kind, "peak_source": csrc,
+                **common}
     return {"bound": "hbm", "achieved": round(gbs, 1), "peak": peaks["hbm"], "unit": "GB/s",
             "frac": round(hbm_frac, 4), "compute_frac": round(c_frac, 4), "compute": kind,
             "peak_source": f"{peaks['src']} HBM copy bandwidth (MEASURED_PEAKS.json hbm_gbs)", **common}
@@ -955,10 +956,9 @@ def main():
                     help="R-ChFSI iterations of the accuracy leg, mixed vs FP64 filter (0: skip)")
     ap.add_argument("--y0-fp32", action="store_true")
     ap.add_argument("--y0-pair32", action="store_true",
-                    help="form step 2 (Y = H X - S X Lambda) in pair-of-FP32 arithmetic in the main measurement")
+                    help="set options.y0_pair32 in the main measurement")
     ap.add_argument("--pair-steps", type=int, default=3,
-                    help="timed calls of the filter with a pair-of-FP32 step 2, reported beside the FP64 one "
-                         "(0: skip)")
+                    help="timed calls of the filter with options.y0_pair32, reported beside the main one (0: skip)")
     ap.add_argument("--no-e2e", action="store_true")
     ap.add_argument("--no-overlap", action="store_true",
                     help="filter the blocks one after another (no overlap of step 2 with the previous block's loop)")
