@@ -18,7 +18,7 @@ class Precision:
     FP32 = 1
     TF32 = 2
     BF16 = 3
-    F32X2 = 4   # FP64 data, pair-of-FP32 arithmetic (apply_H / apply_S)
+    F32X2 = 4   # FP64 data, at least pair-of-FP32 accuracy (apply_H / apply_S)
     names = {"fp64": 0, "fp32": 1, "tf32": 2, "bf16": 3, "f32x2": 4}
 
     @classmethod
