@@ -62,6 +62,13 @@ __device__ __forceinline__ int fx_field(double x) {
   return max((int)((unsigned)__double2hiint(x) >> 20) & 0x7ff, 1);
 }
 
+// the field that a coefficient counts with in the scale of its group: that of |x| with the carry of
+// the low limb's rounding, so that fx_from<63> in the scale leaves a high limb below 2^31
+__device__ __forceinline__ int fx_field_coef(double x) {
+  const long long b = __double_as_longlong(x) & 0x7fffffffffffffffll;
+  return max((int)((b + (1ll << 21)) >> 52), 1);
+}
+
 // x in the unit of a group with the largest exponent field E (E >= fx_field(x), finite), truncated;
 // |x| < 2^(E - 1022) becomes an integer below 2^BITS (54 <= BITS <= 63)
 template <int BITS = FX_F>

@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(fx_threads<NP, VT>(), fx_blocks<NP, VT>()) k_l
     double cm = A.cM;
     if (A.cMcol && v0 + v < A.ncols) cm += A.cMcol[v0 + v];
     cm *= A.mf;
-    const int f = fx_field(cm), scmx = cm == 0.0 ? FX_NONE : f - 1022;
+    const int f = fx_field(cm), scmx = cm == 0.0 ? FX_NONE : fx_field_coef(cm) - 1022;
     const int sv = doV ? A.sV[e] : FX_NONE;
     int D = max(scmx + A.room, doV ? sv - A.zeta : FX_NONE);
     D = max(D, A.hasK ? 0 : -4000);
@@ -597,19 +597,20 @@ __global__ void __launch_bounds__(128) k_wV_fx(int nq, const double *__restrict_
                                                fx2 *__restrict__ out, int *__restrict__ sV) {
   __shared__ int sred[4];
   const size_t e = blockIdx.x;
-  int E = 1, any = 0;
+  int E = 1, any = 0, bad = 0;
   for (int i = threadIdx.x; i < nq; i += 128) {
     const double x = wq[i] * Vq[e * nq + i];
-    E = max(E, fx_field(x));
+    E = max(E, fx_field_coef(x));
     any |= x != 0.0;
+    bad |= fx_field(x) == 0x7ff;
   }
   any = __syncthreads_or(any);
+  bad = __syncthreads_or(bad);
 #pragma unroll
   for (int o = 16; o; o >>= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, o));
   if ((threadIdx.x & 31) == 0) sred[threadIdx.x >> 5] = E;
   __syncthreads();
   E = max(max(sred[0], sred[1]), max(sred[2], sred[3]));
-  const bool bad = E == 0x7ff;
   for (int i = threadIdx.x; i < nq; i += 128) {
     const long long C = bad ? 0 : fx_from<63>(wq[i] * Vq[e * nq + i], E);
     out[e * nq + i] = {fx_hi(C), fx_lo(C)};
