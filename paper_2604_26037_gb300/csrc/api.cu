@@ -1124,11 +1124,11 @@ paw_status paw_destroy(paw_handle c) {
                     &c->DH64, &c->DS64, &c->DSinv64, &c->ws_W, &c->ws_RX,
                     &c->ws_RY, &c->ws_T, &c->ws_Y0f, &c->ws_colscale, &c->ws_red, &c->ws_vec,
                     &c->ws_HX, &c->ws_SX, &c->ws_Hp, &c->ws_Sp, &c->ws_eig, &c->ws_solver, &c->ws_info,
-                    &c->ws_rot, &c->ws_gram, &c->ws_cg, &c->wV, &c->ws_Y0lo, &c->gnb_off, &c->gnb_atom, &c->Gfull, &c->Fsh32, &c->DSinv32,
+                    &c->ws_rot, &c->ws_gram, &c->ws_cg, &c->Vfx, &c->ws_Y0lo, &c->gnb_off, &c->gnb_atom, &c->Gfull, &c->Fsh32, &c->DSinv32,
                     &c->Gfull32, &c->apair_off, &c->apair, &c->nltc.projB, &c->nltc.projBs, &c->nltc.expB, &c->nltc.mdo, &c->nltc.odof, &c->status_dev, &c->proj_ext_dev, &c->own_ngrp,
                     &c->Bk64, &c->Bk32, &c->tc_bk_tf32.He,
                     &c->tc_bk_bf16.He, &c->ws_cx, &c->ws_cy,
-                    &c->nltc.eoff, &c->wVs,
+                    &c->nltc.eoff, &c->Vfx_exp,
                     &c->scr_main.partial, &c->scr_main.pp, &c->scr_main.W2,
                     &c->scr_side.partial, &c->scr_side.pp, &c->scr_side.W2,
                     &c->ws_Y0p[0], &c->ws_Y0p[1], &c->ws_cxp[0], &c->ws_cxp[1], &c->ws_cyp[0], &c->ws_cyp[1], &c->ws_lamp[0], &c->ws_lamp[1], &c->ws_cfp[0], &c->ws_cfp[1]};

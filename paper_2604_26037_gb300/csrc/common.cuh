@@ -177,7 +177,7 @@ struct paw_context {
   // host tables (built by the library's own FE code)
   std::vector<double> K_ref, M_ref, Nq, wq;   // nc*nc, nc*nc, nq*nc, nq
   std::vector<double> gq;                     // (p+2) Gauss nodes on [-1,1]
-  std::vector<double> M1, D1, phiq;           // 1D mass, stiffness ((p+1) Gauss), Lagrange at (p+2) Gauss
+  std::vector<double> M1, D1, phiq, wq1;      // 1D mass, stiffness ((p+1) Gauss), Lagrange at (p+2) Gauss, weights there
 
   // device operator data
   pawfe::DevBuf cell_dofs;   // int32 ncells*nc
@@ -186,10 +186,10 @@ struct paw_context {
   pawfe::DevBuf Me64, Me32, K64;              // nc*nc
   pawfe::DevBuf Nq64, wq64;                   // nq*nc, nq
   pawfe::DevBuf Vq;                           // ncells*nq
-  pawfe::DevBuf wV;                           // ncells*nq: w_q detJ V_q in fixed point (sum-factorised V^e)
-  int wV_valid = 0;
+  pawfe::DevBuf Vfx;                          // ncells*nq: V_q in fixed point (sum-factorised V^e)
+  int Vfx_valid = 0;
   std::shared_ptr<pawfe::SfPlans> sf_plans;   // fixed-point tables of the FP64 operators (sumfac.cu)
-  pawfe::DevBuf wVs;                          // ncells: exponents of wV's fixed-point numbers
+  pawfe::DevBuf Vfx_exp;                      // ncells: exponents of Vfx's numbers
   pawfe::TcMats tc_tf32, tc_bf16;
   pawfe::TcMats tc_bk_tf32, tc_bk_bf16;       // tcgen05 images of B^e (one shared matrix)
   pawfe::NlTcMats nltc;

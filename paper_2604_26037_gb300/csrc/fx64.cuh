@@ -16,11 +16,12 @@
 // sum to 2^-53 of its size, a sum is exact to about one unit in 2^59 of the largest
 // magnitude that its scales allow for.
 //
-// Overflow: the tables that share an accumulator are scaled so that the magnitudes of
-// each of their rows sum to at most 1; in even/odd halves that is a sum of at most 1/2
-// on halves of at most 2^60, so |Y| <= 2^59 whenever |X| <= 2^59.  With |xh| <= 2^28,
-// sum |ch| <= 2^31 and |cl|, |xl| <= 2^31: |hh| <= 2^59 and, over K products between two
-// folds of mm into hh, |mm| <= K 2^59 + 2^62 < 2^63 for K <= 7.
+// Overflow: the magnitudes of each row of a table sum to at most 1; in even/odd halves that is
+// a sum of at most 1/2 on halves of at most 2^60, so a table's results are at most 2^59 where
+// |X| <= 2^59, and a sum of several tables that is contracted again is scaled to that as a whole.
+// With |xh| <= 2^28, sum |ch| <= 2^31 and |cl|, |xl| <= 2^31 the products of one table leave
+// |hh| <= 2^59 and, for up to K = 5 of them, |mm| <= K 2^59 + 2^62 < 2^63; mm is folded into hh before
+// the next table.
 #pragma once
 
 #include <cuda_runtime.h>

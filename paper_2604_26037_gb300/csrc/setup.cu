@@ -183,6 +183,7 @@ void build_tables(paw_context *c) {
   const int nq1 = p + 2, nq = nq1 * nq1 * nq1;
   c->gq = g2;
   c->phiq = phi2;   // phiq[i * np1 + a] = phi_a(g_i)
+  c->wq1 = w2;
   c->Nq.assign((size_t)nq * nc, 0.0);
   c->wq.assign(nq, 0.0);
   for (int q = 0; q < nq; ++q) {
@@ -423,7 +424,7 @@ void rebuild_hamiltonian(paw_context *c) {
   PAW_LAUNCH_CHECK("k_build_He");
   c->tc_tf32.valid = 0;
   c->tc_bf16.valid = 0;
-  c->wV_valid = 0;
+  c->Vfx_valid = 0;
   PAW_CUDA(cudaDeviceSynchronize());
 }
 

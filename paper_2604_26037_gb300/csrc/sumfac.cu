@@ -7,7 +7,8 @@
 // factor into 1D matrices:
 //   K^e = (1/2)(h/2) [D (x) M (x) M + M (x) D (x) M + M (x) M (x) D]   ((p+1)-point Gauss)
 //   M^e = (h/2)^3 M (x) M (x) M
-//   V^e = Phi^T diag(w_q detJ V_q) Phi,  Phi = phi (x) phi (x) phi    ((p+2)-point Gauss)
+//   V^e = (h/2)^3 Psi diag(V_q) Phi,  Phi = phi (x) phi (x) phi, Psi likewise of psi = phi^T diag(w)
+//                                                                     ((p+2)-point Gauss, 1D weights w)
 // with M, D the 1D reference mass and stiffness matrices and phi the Lagrange
 // basis at the 1D Gauss points.  Each application is a chain of 1D
 // contractions of the (p+1)^3 nodal tensor instead of dense products with H^e
@@ -143,20 +144,28 @@ struct Acc {
   }
 };
 
+// Row scales: the rows of M, D, C and psi that belong to node i are divided by 2^tau_i, where
+// 2^tau_i is the size of row i of M.  The rows of a corner node are a tenth of those in the middle
+// of a cell, (1/10)^3 for a corner of the cube, and a result in one common unit would keep that
+// many bits fewer there (largest error of one cell of degree 6, relative to the sum of magnitudes
+// of the entry: S 1.6e-14, with the row scales 2.4e-16, FP64 sums 4.5e-16).  All values of a line
+// carry the factors of the directions already contracted, so that only the exponents of the
+// outputs see them: y at the node (a, b, c) is in units of 2^(tau_a + tau_b + tau_c).
+//
 // Scales, relative to the unit u of the cell's values (|A| the largest row sum of magnitudes
-// of a table A; all chosen on the host):
+// of a table A with its row scales; all chosen on the host):
 //   U after three contractions with phi:            |phi|^3
-//   Z = w V U, aligned for the last stage:          |phi|^3 2^(zeta + D)
+//   Z = V U, aligned for the last stage:            |phi|^3 2^(zeta + D)
 //   P = M x: |M|,  Q = D x: |D|,  S = M P: |M|^2,  R = kD P + kM Q + c S:  rho 2^D
-//   y = fD S + fM R + fB B1:                        2^(eta + D)
-// The kinetic part leaves 1/16 of the range of R to the mass part (c) and 1/4 of that of y to
-// the potential; D (>= 0 with a kinetic part) makes room, per cell and vector, for a
-// coefficient or a potential that is larger.
+//   y = fD S + fM R + fB B1:                        2^(eta + D), each of the three sums at most 1
+// The kinetic part leaves 1/16 of the range of R to the mass part (c); D (>= 0 with a kinetic
+// part) makes room, per cell and vector, for a coefficient or a potential that is larger.
 struct FxLocal {
-  FxEo phi, phit, M, D, kD, kM, fD, fM, fB;
+  FxEo phi, psi, M, D, kD, kM, fD, fM, fB;
+  int tau[9];
   const int *cell_dofs;
-  const fx2 *wV;        // ncells x NQ^3: w_q detJ V_q in the unit of the cell
-  const int *sV;        // ncells: wV is w V 2^-sV (FX_BAD: not finite)
+  const fx2 *V;         // ncells x NQ^3: V_q in the unit of the cell
+  const int *sV;        // ncells: the coefficients are V 2^-(sV + 1) (FX_BAD: not finite)
   const double *X;
   double *Y;
   const double *cMcol;
@@ -164,7 +173,7 @@ struct FxLocal {
   int64_t ldx, ldy;
   int ncols, ntile;
   int hasK, hasM, doV, bad;   // bad: a factor is not finite
-  int room, eta, zeta;   // room: |c| <= 2^-room of the range of R
+  int eta, zeta;
 };
 
 // VT vectors per block, one line of a contraction per thread: the longest stage ((p+2)^2
@@ -185,9 +194,6 @@ template <int NP, int VT>
 constexpr size_t fx_smem() {
   return sizeof(long long) * VT * ((NP + 1) * (NP + 1) * fx_row<NP>() + 2 * NP * NP * fx_rown<NP>());
 }
-// the products of two tables of N1 and N2 columns (and the mass term) need a fold between them
-template <int N1, int N2>
-constexpr bool fx_fold() { return (N1 + 1) / 2 + (N2 + 1) / 2 + (N1 == N2) > 7; }
 template <int NP, int VT>
 constexpr int fx_blocks() { return NP > 7 ? 1 : VT == FX_VT ? 2 : 4; }
 
@@ -251,10 +257,12 @@ __global__ void __launch_bounds__(fx_threads<NP, VT>(), fx_blocks<NP, VT>()) k_l
     double cm = A.cM;
     if (A.cMcol && v0 + v < A.ncols) cm += A.cMcol[v0 + v];
     cm *= A.mf;
-    const int f = fx_field(cm), scmx = cm == 0.0 ? FX_NONE : fx_field_coef(cm) - 1022;
+    // |c| < 2^sc.  The kinetic part takes 15/16 2^-D of the range of R: c has 1/16 where D is 0
+    // and 1/2 (the largest coefficient) from there on
+    const int f = fx_field(cm), sc = cm == 0.0 ? FX_NONE : fx_field_coef(cm) - 1022;
     const int sv = doV ? A.sV[e] : FX_NONE;
-    int D = max(scmx + A.room, doV ? sv - A.zeta : FX_NONE);
-    D = max(D, A.hasK ? 0 : -4000);
+    int D = A.hasK ? (sc <= -4 ? 0 : max(sc + 1, 1)) : max(sc + 1, -4000);
+    if (doV) D = max(D, sv - A.zeta);
     const bool bad = A.bad || f == 0x7ff || sv == FX_BAD;
     sbad[v] = bad;
     if (bad) D = 0;
@@ -305,11 +313,11 @@ __global__ void __launch_bounds__(fx_threads<NP, VT>(), fx_blocks<NP, VT>()) k_l
     }
   }
   __syncthreads();
-  // U3, Z = w V U3 and B2 = phi^T Z: lines along z of W, in registers
+  // U3, Z = V U3 and B2 = psi Z: lines along z of W, in registers
   if (doV && ln < NQ * NQ) {
-    const int2 *wv = reinterpret_cast<const int2 *>(A.wV) + (size_t)e * (NQ * NQ * NQ) + ln;
+    const int2 *Vq = reinterpret_cast<const int2 *>(A.V) + (size_t)e * (NQ * NQ * NQ) + ln;
     const int zs = sZ[v];
-    const long long half = zs > 0 ? 1ll << (zs - 1) : 0;
+    const long long half = zs > 1 ? 1ll << (zs - 2) : 0;
     long long *w = W + ((ln / NQ) * RS + ln % NQ) * VT + v;
     Halves<NP> x;
     x.load(w, NQ * RS * VT);
@@ -330,10 +338,10 @@ __global__ void __launch_bounds__(fx_threads<NP, VT>(), fx_blocks<NP, VT>()) k_l
       }
 #pragma unroll
       for (int t = 0; t < (mid ? 1 : 2); ++t) {
-        const int2 q = __ldg(wv + (t ? NQ - 1 - i : i) * NQ * NQ);
+        const int2 q = __ldg(Vq + (t ? NQ - 1 - i : i) * NQ * NQ);
         long long hh = half, mm = FX_HALF;
         fx_mac(hh, mm, fx_hi(r[t]), fx_lo(r[t]), fx2{q.x, q.y});
-        r[t] = fx_sum(hh, mm) >> zs;
+        r[t] = 2 * fx_sum(hh, mm) >> zs;   // twice the product: coefficients are below 1/2
       }
       if (mid) {
         z.set_e(i, 2 * r[0]);
@@ -344,7 +352,7 @@ __global__ void __launch_bounds__(fx_threads<NP, VT>(), fx_blocks<NP, VT>()) k_l
     }
     Acc<NP> B;
     B.init();
-    B.mac(A.phit, z);
+    B.mac(A.psi, z);
     B.store(w, NQ * RS * VT);
   }
   // S = M P, R = kD P + kM Q + c S: lines along y
@@ -358,7 +366,7 @@ __global__ void __launch_bounds__(fx_threads<NP, VT>(), fx_blocks<NP, VT>()) k_l
     T.init();
     if (A.hasK) {
       T.mac(A.kD, p);
-      if (fx_fold<NP, NP>()) T.fold();
+      T.fold();
       Halves<NP> q;
       q.load(SQ + o, RN * VT);
       T.mac(A.kM, q);
@@ -390,7 +398,7 @@ __global__ void __launch_bounds__(fx_threads<NP, VT>(), fx_blocks<NP, VT>()) k_l
     x.load(w, RS * VT);
     Acc<NP> B;
     B.init();
-    B.mac(A.phit, x);
+    B.mac(A.psi, x);
     B.store(w, RS * VT);
   }
   __syncthreads();
@@ -411,17 +419,18 @@ __global__ void __launch_bounds__(fx_threads<NP, VT>(), fx_blocks<NP, VT>()) k_l
       y.mac(A.fM, r);
     }
     if (doV) {
-      if (fx_fold<NP, NQ>()) y.fold();
+      y.fold();
       Halves<NQ> b;
       b.load(W + ((ln / NP) * NQ + ln % NP) * RS * VT + v, VT);
       y.mac(A.fB, b);
     }
     if (v0 + v < A.ncols) {
-      const int ex = Emax - FX_BIAS + A.eta + D;
+      const int ex = Emax - FX_BIAS + A.eta + D + A.tau[ln % NP] + A.tau[ln / NP];
       const bool bad = Emax == 0x7ff || sbad[v];
       double *Yv = A.Y + v0 + v;
       y.each([&](int a, long long r) {
-        atomicAdd(Yv + sdof[ln * NP + a] * A.ldy, bad ? __longlong_as_double(0x7ff8000000000000ll) : fx_to(r, ex));
+        atomicAdd(Yv + sdof[ln * NP + a] * A.ldy,
+                  bad ? __longlong_as_double(0x7ff8000000000000ll) : fx_to(r, ex + A.tau[a]));
       });
     }
   }
@@ -434,6 +443,7 @@ __global__ void __launch_bounds__(fx_threads<NP, VT>(), fx_blocks<NP, VT>()) k_l
 // C in the place of D; the factors k_x, k_y, k_z, (h/2)^2 and alpha are folded into the tables.
 struct FxBloch {
   FxEo M, C, kyC, kzM, fC, fM;   // z: M, C;  y: M, k_y C, k_z M;  x: alpha (h/2)^2 (k_x C, M)
+  int tau[9];                    // as FxLocal
   const int *cell_dofs;
   const double *X;
   double *Y;
@@ -477,7 +487,7 @@ __global__ void __launch_bounds__(fx_threads<NP, VT>(), fx_blocks<NP, VT>()) k_b
       Acc<NP> T;
       T.init();
       T.mac_anti(A.kyC, p);
-      if (fx_fold<NP, NP>()) T.fold();
+      T.fold();
       Halves<NP> q;
       q.load(SQ + o, RN * VT);
       T.mac(A.kzM, q);
@@ -497,17 +507,17 @@ __global__ void __launch_bounds__(fx_threads<NP, VT>(), fx_blocks<NP, VT>()) k_b
       Halves<NP> s;
       s.load(SX + ln * RN * VT + v, VT);
       y.mac_anti(A.fC, s);
-      if (fx_fold<NP, NP>()) y.fold();
+      y.fold();
     }
     Halves<NP> t;
     t.load(SQ + ln * RN * VT + v, VT);
     y.mac(A.fM, t);
     if (v0 + v < A.ncols) {
-      const int ex = Emax - FX_BIAS + A.eta;
+      const int ex = Emax - FX_BIAS + A.eta + A.tau[ln % NP] + A.tau[ln / NP];
       double *Yv = A.Y + v0 + v;
       y.each([&](int a, long long r) {
         atomicAdd(Yv + sdof[ln * NP + a] * A.ldy,
-                  Emax == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll) : fx_to(r, ex));
+                  Emax == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll) : fx_to(r, ex + A.tau[a]));
       });
     }
   }
@@ -592,14 +602,14 @@ __global__ void __launch_bounds__(fx_threads<NP, VT>(), fx_blocks<NP, VT>())
   }
 }
 
-// w_q detJ V_q of one cell per block in the cell's own unit
-__global__ void __launch_bounds__(128) k_wV_fx(int nq, const double *__restrict__ wq, const double *__restrict__ Vq,
-                                               fx2 *__restrict__ out, int *__restrict__ sV) {
+// V_q of one cell per block in the cell's own unit
+__global__ void __launch_bounds__(128) k_V_fx(int nq, const double *__restrict__ Vq, fx2 *__restrict__ out,
+                                              int *__restrict__ sV) {
   __shared__ int sred[4];
   const size_t e = blockIdx.x;
   int E = 1, any = 0, bad = 0;
   for (int i = threadIdx.x; i < nq; i += 128) {
-    const double x = wq[i] * Vq[e * nq + i];
+    const double x = Vq[e * nq + i];
     E = max(E, fx_field_coef(x));
     any |= x != 0.0;
     bad |= fx_field(x) == 0x7ff;
@@ -612,10 +622,10 @@ __global__ void __launch_bounds__(128) k_wV_fx(int nq, const double *__restrict_
   __syncthreads();
   E = max(max(sred[0], sred[1]), max(sred[2], sred[3]));
   for (int i = threadIdx.x; i < nq; i += 128) {
-    const long long C = bad ? 0 : fx_from<63>(wq[i] * Vq[e * nq + i], E);
+    const long long C = bad ? 0 : fx_from<63>(Vq[e * nq + i], E);
     out[e * nq + i] = {fx_hi(C), fx_lo(C)};
   }
-  if (threadIdx.x == 0) sV[e] = bad ? FX_BAD : any ? E - 1021 : FX_NONE / 2;
+  if (threadIdx.x == 0) sV[e] = bad ? FX_BAD : any ? E - 1022 : FX_NONE / 2;
 }
 
 // even/odd halves of a row-major m x n matrix (see EoMat); the matrix is
@@ -648,20 +658,37 @@ void eo_halves_anti(const double *A, int m, int n, EoMat &out) {
   }
 }
 
-// a 1D matrix, its halves and its largest row sum of magnitudes
+std::vector<double> row_sums(const std::vector<double> &A, int m, int n) {
+  std::vector<double> r(m, 0.0);
+  for (int i = 0; i < m; ++i)
+    for (int j = 0; j < n; ++j) r[i] += std::fabs(A[(size_t)i * n + j]);
+  return r;
+}
+
+// powers of two of the row sums of M relative to the largest, rounded up (a row 1/16 of a power of
+// two above one still counts with it, which doubles no other: degree 8, second node)
+std::vector<int> row_scales(const std::vector<double> &M, int n) {
+  const std::vector<double> r = row_sums(M, n, n);
+  const double top = *std::max_element(r.begin(), r.end());
+  std::vector<int> t(n);
+  for (int i = 0; i < n; ++i) t[i] = (int)std::ceil(std::log2(std::min(r[i], r[n - 1 - i]) / top) - 1.0 / 16);   // 0 .. -3 up to degree 8
+  return t;
+}
+
+// a 1D matrix with its row scales (tau NULL: none), its halves, and its row sums of magnitudes
 struct Tab1 {
   EoMat eo{};
+  std::vector<double> row;
   double norm = 0.0;
-  Tab1(const double *A, int m, int n, bool anti = false) {
+  Tab1(std::vector<double> A, int m, int n, const int *tau, bool anti = false) {
+    for (int i = 0; tau && i < m; ++i)
+      for (int j = 0; j < n; ++j) A[(size_t)i * n + j] = std::ldexp(A[(size_t)i * n + j], -tau[i]);
     if (anti)
-      eo_halves_anti(A, m, n, eo);
+      eo_halves_anti(A.data(), m, n, eo);
     else
-      eo_halves(A, m, n, eo);
-    for (int i = 0; i < m; ++i) {
-      double r = 0.0;
-      for (int j = 0; j < n; ++j) r += std::fabs(A[(size_t)i * n + j]);
-      norm = std::max(norm, r * (1.0 + 1e-6));   // the limbs of A / |A| stay below their limit
-    }
+      eo_halves(A.data(), m, n, eo);
+    row = row_sums(A, m, n);
+    for (double &r : row) norm = std::max(norm, r *= 1.0 + 1e-6);   // the limbs of A / |A| stay below their limit
   }
   // limbs of f A (|f| |A| <= 1)
   void put(FxEo &t, long double f) const {
@@ -729,7 +756,8 @@ void with_sizes(const paw_context *c, int ncols, const char *what, F f) {
 // application takes the GPU.  A bounded number, the oldest is replaced.
 struct SfPlans {
   static constexpr size_t MAX = 4;
-  Tab1 M, D, C, phi, pht;
+  std::vector<int> tau;
+  Tab1 M, D, C, phi, psi;
   struct Local {
     double alpha, cK, cV, cM;
     FxLocal t;
@@ -743,18 +771,28 @@ struct SfPlans {
   size_t next_local = 0, next_bloch = 0;
   FxDensity density{};
 
-  static std::vector<double> transposed(const std::vector<double> &A, int m, int n) {
-    std::vector<double> t((size_t)m * n);
-    for (int i = 0; i < m; ++i)
-      for (int j = 0; j < n; ++j) t[(size_t)j * m + i] = A[(size_t)i * n + j];
+  // psi[a][i] = phi_a(g_i) w_i
+  static std::vector<double> weighted(const paw_context *c) {
+    std::vector<double> t((size_t)c->np1 * c->nq1);
+    for (int i = 0; i < c->nq1; ++i)
+      for (int a = 0; a < c->np1; ++a) t[(size_t)a * c->nq1 + i] = c->phiq[(size_t)i * c->np1 + a] * c->wq1[i];
     return t;
   }
+  // largest |a| (A_b B_c) + |b| (B_b A_c) over two rows b, c: bound of a A (x) B + b B (x) A
+  static long double pair_bound(long double a, long double b, const Tab1 &A, const Tab1 &B) {
+    long double m = 0;
+    for (size_t i = 0; i < A.row.size(); ++i)
+      for (size_t j = 0; j < A.row.size(); ++j)
+        m = std::max(m, std::fabs(a) * A.row[i] * B.row[j] + std::fabs(b) * B.row[i] * A.row[j]);
+    return m;
+  }
   explicit SfPlans(const paw_context *c)
-      : M(c->M1.data(), c->np1, c->np1),
-        D(c->D1.data(), c->np1, c->np1),
-        C(c->C1s.empty() ? c->M1.data() : c->C1s.data(), c->np1, c->np1, true),
-        phi(c->phiq.data(), c->nq1, c->np1),
-        pht(transposed(c->phiq, c->nq1, c->np1).data(), c->np1, c->nq1) {
+      : tau(row_scales(c->M1, c->np1)),
+        M(c->M1, c->np1, c->np1, tau.data()),
+        D(c->D1, c->np1, c->np1, tau.data()),
+        C(c->C1s.empty() ? c->M1 : c->C1s, c->np1, c->np1, tau.data(), true),
+        phi(c->phiq, c->nq1, c->np1, nullptr),
+        psi(weighted(c), c->np1, c->nq1, tau.data()) {
     const long double nP = phi.norm;
     phi.put(density.phi, 1 / nP);
     density.unit = (double)(nP * nP * nP);
@@ -780,8 +818,8 @@ struct SfPlans {
     const double kx = c->kvec[0], ky = c->kvec[1], kz = c->kvec[2];
     // T: k_y C P + k_z M Q in the scale rho, then y = fC S + fM T in the scale 2^eta
     const long double nM = M.norm, nC = C.norm, tiny = 1e-300;
-    const long double rho = std::max(((long double)std::fabs(ky) + std::fabs(kz)) * nC * nM, tiny);
-    const int eta = fx_scale((double)std::max(std::fabs(f) * (std::fabs(kx) * nC * nM * nM + nM * rho), tiny));
+    const long double rho = std::max(pair_bound(ky, kz, C, M), tiny);
+    const int eta = fx_scale((double)std::max(std::fabs(f) * std::max(std::fabs(kx) * nC * nM * nM, nM * rho), tiny));
     M.put(t.M, 1 / nM);
     C.put(t.C, 1 / nC);
     C.put(t.kyC, ky * nM / rho);
@@ -789,6 +827,7 @@ struct SfPlans {
     C.put(t.fC, std::ldexp(f * (kx * nM * nM), -eta));
     M.put(t.fM, std::ldexp(f * rho, -eta));
     t.eta = eta;
+    std::copy(tau.begin(), tau.end(), t.tau);
     Bloch &e = slot(bloch, next_bloch);
     e.alpha = alpha;
     e.t = t;
@@ -805,30 +844,28 @@ struct SfPlans {
     t.doV = cV != 0.0;
     t.bad = !std::isfinite(alpha_in) || !std::isfinite(kf) || !std::isfinite(cV);
     const double alpha = t.bad ? 1.0 : alpha_in;
-    // scales (see FxLocal); without a kinetic part c is a power of two times cM
-    const long double nM = M.norm, nD = D.norm, nP = phi.norm, nT = pht.norm, p3 = nP * nP * nP, akf = std::fabs(kf);
-    const long double rho =
-        t.hasK ? akf * 2 * nD * nM * 16 / 15 : std::ldexp(mf * nM * nM, std::max(fx_scale(cM), -900));
-    t.room = t.hasK ? 4 : 1;
-    t.eta =
-        fx_scale((double)std::max(std::fabs(alpha) * (akf * nD * nM * nM + nM * rho) * (t.doV ? 4 : 3) / 3, tiny));
-    t.zeta = fx_scale((double)(std::ldexp((long double)0.5, t.eta) /
-                               std::max(std::fabs(alpha * cV) * p3 * nT * nT * nT, tiny))) - 1;
-    t.mf = (double)(mf * nM * nM / rho);
+    // scales (see FxLocal); without a kinetic part c is cM / 2 in the scale of cM
+    const long double nM = M.norm, nD = D.norm, nP = phi.norm, nS = psi.norm, p3 = nP * nP * nP, akf = std::fabs(kf);
+    t.mf = (double)(mf * nM * nM / (t.hasK ? pair_bound(kf, kf, D, M) * 16 / 15
+                                           : mf * nM * nM * 2 * std::max(std::fabs(cM) * (1 + 1e-6L), 1e-270L)));
+    const long double rho = mf * nM * nM / t.mf;   // c = cM t.mf has no other rounding
+    t.eta = fx_scale((double)std::max(std::fabs(alpha) * std::max(akf * nD * nM * nM, nM * rho), tiny));
+    const long double fV = alpha * cV * mf * p3 * nS * nS;   // (h/2)^3: detJ
+    t.zeta = fx_scale((double)(std::ldexp((long double)1, t.eta) / std::max(std::fabs(fV) * nS, tiny))) - 1;
     t.cM = cM;
     const Local *near = nullptr;   // tables of another alpha: only the last stage differs
     for (const Local &e : local)
       if (e.cK == cK && e.cV == cV && e.cM == cM && !e.t.bad) near = &e;
     if (near) {
       t.phi = near->t.phi;
-      t.phit = near->t.phit;
+      t.psi = near->t.psi;
       t.M = near->t.M;
       t.D = near->t.D;
       t.kD = near->t.kD;
       t.kM = near->t.kM;
     } else {
       phi.put(t.phi, 1 / nP);
-      pht.put(t.phit, 1 / nT);
+      psi.put(t.psi, 1 / nS);
       M.put(t.M, 1 / nM);
       D.put(t.D, 1 / nD);
       D.put(t.kD, kf * nM / rho);
@@ -836,7 +873,8 @@ struct SfPlans {
     }
     D.put(t.fD, std::ldexp(alpha * (kf * nM * nM), -t.eta));
     M.put(t.fM, std::ldexp(alpha * rho, -t.eta));
-    pht.put(t.fB, t.doV ? std::ldexp(alpha * (cV * p3 * nT * nT), t.zeta - t.eta) : 0);
+    psi.put(t.fB, t.doV ? std::ldexp(fV, t.zeta - t.eta) : 0);
+    std::copy(tau.begin(), tau.end(), t.tau);
     Local &e = slot(local, next_local);
     e.alpha = alpha_in;
     e.cK = cK;
@@ -888,18 +926,17 @@ void local_sf(paw_context *c, const double *X, int ldx, double *Y, int ldy, int 
               double cV, double cM, const double *cMcol, cudaStream_t s) {
   if (ncols <= 0) return;
   FxLocal t = plans(c).local_tables(c, alpha, cK, cV, cM);
-  // w_q V_q per cell (rebuilt lazily after a potential change)
-  if (!c->wV_valid) {
-    c->wV.ensure(sizeof(fx2) * (size_t)c->ncells * c->nq, &c->dev_bytes);
-    c->wVs.ensure(sizeof(int) * (size_t)c->ncells, &c->dev_bytes);
-    k_wV_fx<<<(unsigned)c->ncells, 128, 0, s>>>(c->nq, c->wq64.as<double>(), c->Vq.as<double>(), c->wV.as<fx2>(),
-                                                 c->wVs.as<int>());
-    PAW_LAUNCH_CHECK("k_wV_fx");
-    c->wV_valid = 1;
+  // V_q per cell (rebuilt lazily after a potential change)
+  if (!c->Vfx_valid) {
+    c->Vfx.ensure(sizeof(fx2) * (size_t)c->ncells * c->nq, &c->dev_bytes);
+    c->Vfx_exp.ensure(sizeof(int) * (size_t)c->ncells, &c->dev_bytes);
+    k_V_fx<<<(unsigned)c->ncells, 128, 0, s>>>(c->nq, c->Vq.as<double>(), c->Vfx.as<fx2>(), c->Vfx_exp.as<int>());
+    PAW_LAUNCH_CHECK("k_V_fx");
+    c->Vfx_valid = 1;
   }
   t.cell_dofs = c->cell_dofs.as<int>();
-  t.wV = c->wV.as<fx2>();
-  t.sV = c->wVs.as<int>();
+  t.V = c->Vfx.as<fx2>();
+  t.sV = c->Vfx_exp.as<int>();
   t.X = X;
   t.Y = Y;
   t.cMcol = cMcol;

@@ -30,3 +30,41 @@ def test_point_potentials_just_below_a_power_of_two(p, size):
     fe.set_veff(torch.from_numpy(V).cuda())
     assert rel_err(fe.apply_H(to_dev(X)).cpu().numpy(), O.PawOperators(_system(p), Vq=V).apply_H(X)) < TOL
     fe.close()
+
+
+@pytest.mark.parametrize("p", [2, 4, 6, 8])
+def test_small_entries_at_cell_corners(p):
+    """Errors relative to each entry, down to the corners of a cell, whose rows are far smaller than
+    those in its middle.  A product vector f(x) f(y) f(z) inside one cell gives S X = mu mu mu and
+    K X = delta mu mu + mu delta mu + mu mu delta there, so the lines through the middle node predict every
+    other entry, whatever the 1D matrices are.
+
+    Tolerance: three to five contractions, each exact to two units of 2^-59 of the scaled range,
+    of which an entry takes at least 2^-5 (2^-3 for the row sizes left by the row scales, 2^-2 for the
+    others): 10 * 2^-59 * 2^5 = 5.6e-16, with the rounding of the output 7e-16; a prediction uses four
+    such entries besides its own: 3.5e-15 of the sum of magnitudes."""
+    import torch
+    import paper_2604_26037_gb300 as P
+    from oracle import fe as F
+    s = dict(_system(p), natoms=0, positions=np.zeros((0, 3)), D=None, dS=None)
+    fe = P.PawFE.from_system(s)
+    N1, n, m, ncol, tol = 3 * p, p + 1, p // 2, 40, 3.5e-15
+    fe.set_veff(torch.zeros((27, (p + 2) ** 3), dtype=torch.float64, device="cuda"))
+    f = np.zeros((N1, ncol))
+    f[1:p] = np.random.default_rng(p).integers(2 ** 16, 2 ** 17, (p - 1, ncol)) * (-1.0) ** np.arange(p - 1)[:, None]
+    X = np.einsum("kv,jv,iv->kjiv", f, f, f).reshape(-1, ncol)       # 51 bits: exact
+    S, H = (c(to_dev(X)).cpu().numpy().reshape(N1, N1, N1, ncol)[:n, :n, :n].astype(np.longdouble)
+            for c in (fe.apply_S, fe.apply_H))
+    fe.close()
+    x = F.Mesh(7.5, 3, p).xi
+    M = np.einsum("q,qa,qb->ab", F.gauss_rule(n)[1], *2 * [F.lagrange(x, F.gauss_rule(n)[0])[0]])
+    mu = [S[:, m, m] / S[m, m, m], S[m, :, m] / S[m, m, m], S[m, m, :] / S[m, m, m]]
+    am = [np.abs(M) @ np.abs(f[:n]) / np.abs(M[m] @ f[:n])] * 3     # sums of magnitudes of mu
+    line = lambda a, b, c: np.einsum("kv,jv,iv->kjiv", a, b, c)
+    assert (np.abs(S - line(*mu) * S[m, m, m]) / np.abs(line(*am) * S[m, m, m])).max() < tol
+    d0 = H[m, m, m] / 3
+    Hm = [H[:, m, m], H[m, :, m], H[m, m, :]]
+    de = [h - 2 * u * d0 for h, u in zip(Hm, mu)]
+    ad = [np.abs(h) + 2 * u * np.abs(d0) for h, u in zip(Hm, am)]
+    three = lambda d, u: line(d[0], u[1], u[2]) + line(u[0], d[1], u[2]) + line(u[0], u[1], d[2])
+    assert (np.abs(H - three(de, mu)) / three(ad, am)).max() < tol
