@@ -82,7 +82,18 @@ __device__ __forceinline__ long long fx_from(double x, int E) {
   return (int)hi < 0 ? -t : t;
 }
 
-// the same for FP32 numbers (fields of the equal FP64 numbers)
+// the same rounded to nearest (ties away from zero), |result| <= 2^BITS (53 <= BITS <= 61)
+template <int BITS>
+__device__ __forceinline__ long long fx_round(double x, int E) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const int f = (int)(hi >> 20) & 0x7ff;
+  const unsigned mh = (hi & 0xfffffu) | (f ? 0x100000u : 0u);
+  const unsigned long long m = ((unsigned long long)mh << 32 | lo) << (BITS - 52);
+  const long long t = (long long)(((m >> min(E - max(f, 1), 63)) + 1) >> 1);
+  return (int)hi < 0 ? -t : t;
+}
+
+// fx_field and fx_from for FP32 numbers (fields of the equal FP64 numbers)
 __device__ __forceinline__ int fx_field(float x) {
   const int f = (int)(__float_as_uint(x) >> 23) & 0xff;
   return f == 0xff ? 0x7ff : max(f, 1) + 896;

@@ -6,13 +6,17 @@
 // GB300 retires 2 FP64 FMAs per clock and SM and 1024 products of an FP16 mma.sync.  Each
 // operand is scaled by a power of two per column (P: per pair and projector; X: per vector over
 // the owned nodes of the cell; W: per vector over the coefficients that reach the cell), rounded
-// to a 55-bit integer and written in seven balanced digits of radix 256, each exact in FP16.
-// Products of digits i and j (0 = lowest) with i + j >= 5 are summed by i + j in FP32
+// to an integer of at most 2^54 and written in seven balanced digits of radix 256, each exact in
+// FP16 (the error-free splitting of Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59, 2012, with
+// fixed digits).  Products of digits i and j (0 = lowest) with i + j >= 5 are summed by i + j in FP32
 // accumulators: at most seven products of magnitude 2^14 share one and at most 144 terms are
 // summed between two flushes, 2^14 * 7 * 144 < 2^24, so every accumulator holds an exact
-// integer.  A flush adds the eight accumulators into one 64-bit sum.  What is left out (i + j
-// <= 4) is below 2^-58 of the largest product, and the rounding of the operands 2^-55 of their
-// column's largest entry, which is no more than the rounding of an FP64 sum over the nodes.
+// integer.  A flush rounds the eight accumulators into one 64-bit sum.  What is left out (i + j
+// <= 4) is below 2^-58 of the largest product, the rounding of the operands at most 2^-54 of their
+// column's largest entry, and the rounding of a flush 2^-(61 - b) of the product of the two columns' units
+// for at most 2^b terms.  Errors relative to the sum of the magnitudes, from a model of these sums: 216
+// terms of like size 1.1e-17 (rms; FP64 sums 5.5e-17), 6144 terms 3.3e-17 (5.0e-17); with operands and
+// flushes cut off instead of rounded 2.0e-17 and 9.1e-16.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -26,7 +30,7 @@ namespace pawfe {
 namespace {
 
 constexpr int DG = 7;            // digits of an operand
-constexpr int DG_BITS = 54;      // |integer| < 2^54: the top digit stays within +-65
+constexpr int DG_BITS = 54;      // |integer| <= 2^54: the top digit stays within +-65
 constexpr int DG_SUMS = 8;       // accumulators: digit positions 5 .. 12
 constexpr int FLUSH = 9;         // k steps of 16 between two flushes
 // coefficients of one batch of the expansion: 8 k steps, or 7 where sums of several batches share
@@ -124,7 +128,7 @@ struct Tile {
           if (i + j >= 5) mma16(c[n][i + j - 5], a[i], b[j][0], b[j][1]);
     }
   }
-  // s += the accumulators in units of 2^(72 - sh) (operand units), accumulators cleared
+  // s += the accumulators in units of 2^(72 - sh) (operand units), rounded; accumulators cleared
   __device__ __forceinline__ void flush(int sh) {
 #pragma unroll
     for (int n = 0; n < 2; ++n)
@@ -139,17 +143,17 @@ struct Tile {
         fx_mad(hi, dig(6), 1 << 16);
         fx_mad(hi, dig(7), 1 << 24);
         hi += lo >> 32;
-        s[n][i] += (long long)((unsigned long long)hi << sh | (unsigned)lo >> (32 - sh));
+        s[n][i] += (long long)((unsigned long long)hi << sh) + ((((unsigned)lo >> (31 - sh)) + 1) >> 1);
       }
     clear();
   }
 };
 
-// bits left for the sums: |sum| < 2^(36 + log2 K) units of 2^72
+// bits left for the sums: |sum| <= 2^(36 + log2 K) units of 2^72, 2^62 units of 2^(72 - sh)
 __host__ __device__ __forceinline__ int sum_shift(int K) {
   int b = 0;
   while ((1 << b) < K) ++b;
-  return 25 - b;
+  return 26 - b;
 }
 
 struct FxNl {
@@ -252,8 +256,8 @@ __global__ void __launch_bounds__(256, 2) k_fx_project(FxNl A, const double *__r
     E[0] = Em[2 * vp];
     E[1] = Em[2 * vp + 1];
     auto put = [&](int o, double a, double b) {
-      store_digits(sm, plane, piece<VT>(o, vp >> 2) + (vp & 3) * 4, fx_from<DG_BITS>(a, E[0]),
-                   fx_from<DG_BITS>(b, E[1]));
+      store_digits(sm, plane, piece<VT>(o, vp >> 2) + (vp & 3) * 4, fx_round<DG_BITS>(a, E[0]),
+                   fx_round<DG_BITS>(b, E[1]));
     };
 #pragma unroll
     for (int i = 0; i < NR; ++i)
@@ -360,8 +364,8 @@ __global__ void __launch_bounds__(256, 2) k_fx_expand(FxNl N, ExpArgs A, const d
         get(W, b * BP * NPAD + r, x, y);
         const int s = N.sP[((size_t)k0 + b * BP) * NPAD + r];
         store_digits(sm, plane, piece<VT>(r, vp >> 2) + (vp & 3) * 4,
-                     x == 0.0 ? 0 : fx_from<DG_BITS>(x, Em[w][2 * vp] - s),
-                     y == 0.0 ? 0 : fx_from<DG_BITS>(y, Em[w][2 * vp + 1] - s));
+                     x == 0.0 ? 0 : fx_round<DG_BITS>(x, Em[w][2 * vp] - s),
+                     y == 0.0 ? 0 : fx_round<DG_BITS>(y, Em[w][2 * vp + 1] - s));
       }
       __syncthreads();
       for (int u = warp; u < units; u += 8) {
@@ -448,7 +452,7 @@ __global__ void __launch_bounds__(128) k_build_digits(int own, int kt, int npad,
   if (threadIdx.x == 0) mask[k] = ms;
   for (int i = threadIdx.x; i < kt * 16 * npad; i += 128) {
     const int o = i / npad, al = i % npad;
-    const long long V = o < own ? fx_from<DG_BITS>(Pk[(size_t)o * npad + al], E[al]) : 0;
+    const long long V = o < own ? fx_round<DG_BITS>(Pk[(size_t)o * npad + al], E[al]) : 0;
     const unsigned long long bytes = (unsigned long long)V + DG_BIAS;
     // element (r, c) of a 16 x 16 A tile: lane, byte of its eight
     auto put = [&](unsigned char *img, int r, int c) {

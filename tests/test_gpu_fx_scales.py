@@ -6,6 +6,7 @@ import numpy as np
 import pytest
 
 from tests.gpu_util import rel_err, to_dev
+from tests.oracle_systems import mini_system, sym_random
 from tests.test_gpu_local_fx import TOL, _fe, _oracle, _system
 
 pytestmark = pytest.mark.gpu
@@ -68,3 +69,19 @@ def test_small_entries_at_cell_corners(p):
     ad = [np.abs(h) + 2 * u * np.abs(d0) for h, u in zip(Hm, am)]
     three = lambda d, u: line(d[0], u[1], u[2]) + line(u[0], d[1], u[2]) + line(u[0], u[1], d[2])
     assert (np.abs(H - three(de, mu)) / three(ad, am)).max() < tol
+
+
+def test_many_coefficients_of_both_signs():
+    """S (-X) = -S X with 190 atoms on every cell: coefficients of 64 batches, whose sums are rounded
+    one by one into 64 bits.  Rounding to nearest has no sign: what is left are FP64 additions of the
+    eight cells of a node in another order, 16 * 2^-53 of the largest entry of a column."""
+    import paper_2604_26037_gb300 as P
+    rng = np.random.default_rng(12)
+    s = mini_system(L=5.0, n=2, p=3, positions=rng.uniform(0.0, 5.0, (190, 3)),
+                    shells=[(0, 0.36), (0, 0.3), (1, 0.36), (1, 0.33), (2, 0.36), (2, 0.3)],
+                    D=sym_random(rng, 190, 18, 0.1), dS=sym_random(rng, 190, 18, 0.01), vdepth=1.0)
+    fe = P.PawFE.from_system(s)
+    X = to_dev(rng.standard_normal((fe.ndof, 33)))
+    Y, Z = fe.apply_S(X).cpu().numpy(), fe.apply_S(-X).cpu().numpy()
+    fe.close()
+    assert (np.abs(Y + Z).max(0) / np.abs(Y).max(0)).max() <= 16 * 2.0 ** -53
