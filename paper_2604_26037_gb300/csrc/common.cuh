@@ -212,8 +212,9 @@ struct paw_context {
   pawfe::DevBuf ownP32;                       // nown_pairs * own * npad
   pawfe::DevBuf own_ngrp;                     // int32 per pair: projector groups of 4 with a nonzero value
   // FP64 contractions (nonlocal_fx.cu): digit images of P for the projection and the
-  // expansion, exponent per pair and projector, node tiles with nonzero values per pair
-  pawfe::DevBuf own_proj_dg, own_exp_dg, own_sP, own_mask;
+  // expansion, exponent per pair and projector, node tiles with nonzero values per pair, row
+  // exponents per cell and owned node (int16)
+  pawfe::DevBuf own_proj_dg, own_exp_dg, own_sP, own_mask, own_r;
   int64_t proj_nnz = 0;                       // nonzero (owned node, projector) entries over all pairs
   pawfe::DevBuf apair_off, apair;             // atom-major list of the pairs (int32)
   // atom-pair Gram blocks G_ab = P^a^T M_D^-1 P^b for atoms with common support

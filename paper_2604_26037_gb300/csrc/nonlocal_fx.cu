@@ -3,9 +3,12 @@
 //   projection  U[k][al][v] = sum_o P[k][o][al] s(o) X[o][v]          per owner pair k
 //   expansion   S[o][v]     = sum_k sum_al P[k][o][al] W[a_k][al][v]  with the output stage of its mode
 //
-// GB300 retires 2 FP64 FMAs per clock and SM and 1024 products of an FP16 mma.sync.  Each
-// operand is scaled by a power of two per column (P: per pair and projector; X: per vector over
-// the owned nodes of the cell; W: per vector over the coefficients that reach the cell), rounded
+// GB300 retires 2 FP64 FMAs per clock and SM and 1024 products of an FP16 mma.sync.  Rows first: a
+// projector falls by 1e-8 to its cut-off, so row o of P is divided by 2^r(o), the size of its
+// largest entry over the pairs of the cell, X(o) is multiplied by it, and the sums of the
+// expansion take it back; an X that grows where P falls then keeps its bits where the
+// products are large.  Each operand is then scaled by a power of two per column (P: per pair and projector;
+// X: per vector over the owned nodes of the cell; W: per vector over the coefficients that reach the cell), rounded
 // to an integer of at most 2^54 and written in seven balanced digits of radix 256, each exact in
 // FP16 (the error-free splitting of Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59, 2012, with
 // fixed digits).  Products of digits i and j (0 = lowest) with i + j >= 5 are summed by i + j in FP32
@@ -16,7 +19,8 @@
 // column's largest entry, and the rounding of a flush 2^-(61 - b) of the product of the two columns' units
 // for at most 2^b terms.  Errors relative to the sum of the magnitudes, from a model of these sums: 216
 // terms of like size 1.1e-17 (rms; FP64 sums 5.5e-17), 6144 terms 3.3e-17 (5.0e-17); with operands and
-// flushes cut off instead of rounded 2.0e-17 and 9.1e-16.
+// flushes cut off instead of rounded 2.0e-17 and 9.1e-16.  X falling by e^-18 over 216 nodes while P
+// grows by as much: 3.2e-17 (FP64 5.1e-17; without the row factors 7.9e-11).
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -36,6 +40,8 @@ constexpr int FLUSH = 9;         // k steps of 16 between two flushes
 // coefficients of one batch of the expansion: 8 k steps, or 7 where sums of several batches share
 // the shared memory (two blocks per SM at degree 6)
 constexpr int EXP_K = 128, EXP_K_MANY = 112;
+constexpr int NODE_OFF = -8192;   // row exponent of a node on which every projector of the cell is zero
+constexpr int NONFINITE = 1 << 20;   // column exponent that marks an infinity or a NaN
 constexpr unsigned long long DG_BIAS = 0x80808080808080ull;
 
 // rows (nodes or coefficients) of VT FP16 digits; the 16-byte pieces of a row are placed so
@@ -161,7 +167,8 @@ struct FxNl {
   int bp;                         // pairs of one batch of the expansion
   const int *own_off, *own_atom;
   const unsigned char *proj, *exp;   // digit images (operand A of the projection, of the expansion)
-  const int *sP;                  // exponent per pair and projector: |P| < 2^sP
+  const int *sP;                  // exponent per pair and projector: |P(o) 2^-r(o)| < 2^sP
+  const short *r;                 // ncells x own: row exponents (NODE_OFF: P is zero there)
   const unsigned *mask;           // per pair: bit t set when a node of tile t has a nonzero value
 };
 
@@ -207,6 +214,7 @@ __global__ void __launch_bounds__(256, 2) k_fx_project(FxNl A, const double *__r
   constexpr int MT = NPAD / 16, H = VT / 16, VP = VT / 2, ROWS = 256 / VP;
   extern __shared__ __align__(128) unsigned char sm[];
   __shared__ int ooff[512];
+  __shared__ short rs[512];
   __shared__ int red[8 * VT], Em[VT];
   const int ntile = (ncols + VT - 1) / VT;
   const int e = blockIdx.x / ntile, v0 = (blockIdx.x - e * ntile) * VT;
@@ -214,7 +222,10 @@ __global__ void __launch_bounds__(256, 2) k_fx_project(FxNl A, const double *__r
   if (k0 == k1) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int own = A.own, plane = A.kt * 16 * VT * 2;
-  for (int o = tid; o < own; o += 256) ooff[o] = owned_offset(o, A.p, A.N1);
+  for (int o = tid; o < own; o += 256) {
+    ooff[o] = owned_offset(o, A.p, A.N1);
+    rs[o] = A.r[(size_t)e * own + o];
+  }
   const int64_t base = owned_base(e, A.n, A.p, A.N1);
   __syncthreads();
   {
@@ -231,11 +242,16 @@ __global__ void __launch_bounds__(256, 2) k_fx_project(FxNl A, const double *__r
         y *= m;
       }
     };
+    // exponent that a value counts with; what stands on a node without projectors does not enter
+    auto field = [&](double x, int o) {
+      const int f = fx_field(x), r = rs[o];
+      return f == 0x7ff && r != NODE_OFF ? NONFINITE : f + r;
+    };
     // the values of the first NR rows of the thread (all of them up to degree 6) stay in
     // registers between the maxima and the digits
     constexpr int NR = 14;
     double x[NR], y[NR];
-    int E[2] = {1, 1};
+    int E[2] = {NODE_OFF / 2, NODE_OFF / 2};
 #pragma unroll
     for (int i = 0; i < NR; ++i) {
       x[i] = y[i] = 0.0;
@@ -244,20 +260,22 @@ __global__ void __launch_bounds__(256, 2) k_fx_project(FxNl A, const double *__r
     for (int o = r0 + NR * ROWS; o < own; o += ROWS) {
       double a, b;
       get(o, a, b);
-      E[0] = max(E[0], fx_field(a));
-      E[1] = max(E[1], fx_field(b));
+      E[0] = max(E[0], field(a, o));
+      E[1] = max(E[1], field(b, o));
     }
 #pragma unroll
-    for (int i = 0; i < NR; ++i) {
-      E[0] = max(E[0], fx_field(x[i]));
-      E[1] = max(E[1], fx_field(y[i]));
-    }
+    for (int i = 0; i < NR; ++i)
+      if (r0 + i * ROWS < own) {
+        E[0] = max(E[0], field(x[i], r0 + i * ROWS));
+        E[1] = max(E[1], field(y[i], r0 + i * ROWS));
+      }
     max_of_vectors<VT>(E, red, Em);
     E[0] = Em[2 * vp];
     E[1] = Em[2 * vp + 1];
     auto put = [&](int o, double a, double b) {
-      store_digits(sm, plane, piece<VT>(o, vp >> 2) + (vp & 3) * 4, fx_round<DG_BITS>(a, E[0]),
-                   fx_round<DG_BITS>(b, E[1]));
+      const int r = o < own ? rs[o] : 0;
+      store_digits(sm, plane, piece<VT>(o, vp >> 2) + (vp & 3) * 4, a == 0.0 ? 0 : fx_round<DG_BITS>(a, E[0] - r),
+                   b == 0.0 ? 0 : fx_round<DG_BITS>(b, E[1] - r));
     };
 #pragma unroll
     for (int i = 0; i < NR; ++i)
@@ -301,8 +319,8 @@ __global__ void __launch_bounds__(256, 2) k_fx_project(FxNl A, const double *__r
         for (int j = 0; j < 2; ++j) {
           const int l = half * 16 + n * 8 + 2 * (lane & 3) + j, v = v0 + l;
           if (v < ncols)
-            Uk[v] = Em[l] == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll)
-                                   : fx_to_small(t.s[n][2 * r + j], ex + Em[l]);
+            Uk[v] = Em[l] >= NONFINITE ? __longlong_as_double(0x7ff8000000000000ll)
+                                       : fx_to_small(t.s[n][2 * r + j], ex + Em[l]);
         }
     }
   }
@@ -320,15 +338,19 @@ template <int NPAD, int VT, int MODE>
 __global__ void __launch_bounds__(256, 2) k_fx_expand(FxNl N, ExpArgs A, const double *__restrict__ W1,
                                                       const double *__restrict__ W2) {
   constexpr int MT = NPAD / 16, H = VT / 16, VP = VT / 2, ROWS = 256 / VP;
-  constexpr int NW = (MODE == EXP_RECURRENCE) ? 2 : 1, BIG = 1 << 20;
+  constexpr int NW = (MODE == EXP_RECURRENCE) ? 2 : 1;
   const int BP = N.bp, plane = BP * NPAD * VT * 2;
   extern __shared__ __align__(128) unsigned char sm[];
   __shared__ int red[8 * VT], Em[NW][VT], ooff[512];
+  __shared__ short rs[512];
   const int ncols = A.ncols, ntile = (ncols + VT - 1) / VT;
   const int e = blockIdx.x / ntile, v0 = (blockIdx.x - e * ntile) * VT;
   const int k0 = N.own_off[e], np = N.own_off[e + 1] - k0;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, own = N.own;
-  for (int o = tid; o < own; o += 256) ooff[o] = owned_offset(o, N.p, N.N1);   // (synchronised with the maxima)
+  for (int o = tid; o < own; o += 256) {   // (synchronised with the maxima)
+    ooff[o] = owned_offset(o, N.p, N.N1);
+    rs[o] = np ? N.r[(size_t)e * own + o] : NODE_OFF;
+  }
   const int vp = tid % VP, r0 = tid / VP;
   const bool ok0 = v0 + 2 * vp < ncols, ok1 = v0 + 2 * vp + 1 < ncols;
   // W of row r (pair r / NPAD of the cell, projector r % NPAD), 0 where there is none
@@ -339,13 +361,13 @@ __global__ void __launch_bounds__(256, 2) k_fx_expand(FxNl N, ExpArgs A, const d
   };
   for (int w = 0; w < NW; ++w) {
     const double *W = w ? W2 : W1;
-    int E[2] = {-BIG, -BIG};
+    int E[2] = {-NONFINITE, -NONFINITE};
     for (int r = r0; r < np * NPAD; r += ROWS) {
       double x, y;
       get(W, r, x, y);
       const int s = N.sP[(size_t)k0 * NPAD + r], fx = fx_field(x), fy = fx_field(y);
-      if (x != 0.0) E[0] = max(E[0], fx == 0x7ff ? BIG : fx + s);
-      if (y != 0.0) E[1] = max(E[1], fy == 0x7ff ? BIG : fy + s);
+      if (x != 0.0) E[0] = max(E[0], fx == 0x7ff ? NONFINITE : fx + s);
+      if (y != 0.0) E[1] = max(E[1], fy == 0x7ff ? NONFINITE : fy + s);
     }
     max_of_vectors<VT>(E, red, Em[w]);
   }
@@ -388,8 +410,9 @@ __global__ void __launch_bounds__(256, 2) k_fx_expand(FxNl N, ExpArgs A, const d
         t.flush(sh);
         const bool last = b + 1 == nbatch;
         const int l0 = half * 16 + 2 * (lane & 3), e0 = 72 - sh - 2 * DG_BITS - 1022;
-        auto value = [&](long long y, int E) {
-          return E >= BIG ? __longlong_as_double(0x7ff8000000000000ll) : fx_to_small(y, e0 + E);
+        auto value = [&](long long y, int E, int r) {
+          if (E >= NONFINITE) return r == NODE_OFF ? 0.0 : __longlong_as_double(0x7ff8000000000000ll);
+          return fx_to_small(y, e0 + E + r);
         };
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
@@ -405,6 +428,7 @@ __global__ void __launch_bounds__(256, 2) k_fx_expand(FxNl N, ExpArgs A, const d
           }
           if (o >= own) continue;
           const int64_t d = base + ooff[o];
+          const int ro = rs[o];
           const double m = MODE == EXP_SET ? 0.0 : static_cast<const double *>(A.mdinv)[d];
           double *Y = static_cast<double *>(A.Y) + d * A.ldy + v0 + l0;
           const double *Xi = MODE == EXP_SET ? nullptr : static_cast<const double *>(A.Xin) + d * A.ldx + v0 + l0;
@@ -414,14 +438,14 @@ __global__ void __launch_bounds__(256, 2) k_fx_expand(FxNl N, ExpArgs A, const d
             if (v0 + l0 + c >= ncols) continue;
             const long long s = t.s[i >> 1][2 * r + (i & 1)];
             if (MODE == EXP_SET) {
-              Y[c] = value(s, Em[0][l0 + c]);
+              Y[c] = value(s, Em[0][l0 + c], ro);
             } else if (MODE == EXP_SINV) {
-              Y[c] = m * (Xi[c] - value(s, Em[0][l0 + c]));
+              Y[c] = m * (Xi[c] - value(s, Em[0][l0 + c], ro));
             } else if (w == 0) {
-              Y[c] = m * (Xi[c] - value(s, Em[0][l0 + c]));
+              Y[c] = m * (Xi[c] - value(s, Em[0][l0 + c], ro));
             } else {
               double *RX = static_cast<double *>(A.RX) + d * A.ldx + v0 + l0 + c;
-              const double bracket = -A.beta * Xi[c] - A.gamma * *RX + value(s, Em[NW - 1][l0 + c]);
+              const double bracket = -A.beta * Xi[c] - A.gamma * *RX + value(s, Em[NW - 1][l0 + c], ro);
               *RX = fma(A.c64[v0 + l0 + c], static_cast<const double *>(A.Y0)[d * A.ldy0 + v0 + l0 + c], bracket);
             }
           }
@@ -431,28 +455,54 @@ __global__ void __launch_bounds__(256, 2) k_fx_expand(FxNl N, ExpArgs A, const d
   }
 }
 
+// row exponents of one cell per block: that of the largest entry of the row over the cell's pairs
+__global__ void __launch_bounds__(128) k_node_scales(int own, int npad, const int *__restrict__ own_off,
+                                                     const double *__restrict__ P, short *__restrict__ r) {
+  const int e = blockIdx.x, k0 = own_off[e], k1 = own_off[e + 1];
+  for (int o = threadIdx.x; o < own; o += 128) {
+    int f = NODE_OFF;
+    for (int k = k0; k < k1; ++k)
+      for (int al = 0; al < npad; ++al) {
+        const double x = P[((size_t)k * own + o) * npad + al];
+        if (x != 0.0) f = max(f, fx_field(x) - 1022);
+      }
+    r[(size_t)e * own + o] = (short)f;
+  }
+}
+
 // digit images, exponents and node-tile masks of one pair per block
-__global__ void __launch_bounds__(128) k_build_digits(int own, int kt, int npad, const double *__restrict__ P,
-                                                      unsigned char *__restrict__ proj, unsigned char *__restrict__ exp,
-                                                      int *__restrict__ sP, unsigned *__restrict__ mask) {
+__global__ void __launch_bounds__(128) k_build_digits(int ncells, int own, int kt, int npad,
+                                                      const int *__restrict__ own_off, const double *__restrict__ P,
+                                                      const short *__restrict__ r, unsigned char *__restrict__ proj,
+                                                      unsigned char *__restrict__ exp, int *__restrict__ sP,
+                                                      unsigned *__restrict__ mask) {
   __shared__ int E[32];
   __shared__ unsigned ms;
   const size_t k = blockIdx.x;
+  int e = 0;   // cell of the pair: own_off[e] <= k < own_off[e + 1]
+  for (int n = ncells; n > 1;) {
+    const int h = n / 2;
+    if (own_off[e + h] <= (int)k) e += h, n -= h;
+    else n = h;
+  }
+  const short *rs = r + (size_t)e * own;
   const int mt = npad / 16;
   const double *Pk = P + k * own * npad;
-  if (threadIdx.x < 32) E[threadIdx.x] = 1;
+  if (threadIdx.x < 32) E[threadIdx.x] = NODE_OFF / 2;
   if (threadIdx.x == 0) ms = 0;
   __syncthreads();
   for (int i = threadIdx.x; i < own * npad; i += 128) {
-    atomicMax(&E[i % npad], fx_field(Pk[i]));
-    if (Pk[i] != 0.0) atomicOr(&ms, 1u << (i / npad / 16));
+    if (Pk[i] == 0.0) continue;
+    atomicMax(&E[i % npad], fx_field(Pk[i]) - rs[i / npad]);
+    atomicOr(&ms, 1u << (i / npad / 16));
   }
   __syncthreads();
   if (threadIdx.x < npad) sP[k * npad + threadIdx.x] = E[threadIdx.x] - 1022;
   if (threadIdx.x == 0) mask[k] = ms;
   for (int i = threadIdx.x; i < kt * 16 * npad; i += 128) {
     const int o = i / npad, al = i % npad;
-    const long long V = o < own ? fx_round<DG_BITS>(Pk[(size_t)o * npad + al], E[al]) : 0;
+    const double x = o < own ? Pk[(size_t)o * npad + al] : 0.0;
+    const long long V = x == 0.0 ? 0 : fx_round<DG_BITS>(x, E[al] + rs[o]);
     const unsigned long long bytes = (unsigned long long)V + DG_BIAS;
     // element (r, c) of a 16 x 16 A tile: lane, byte of its eight
     auto put = [&](unsigned char *img, int r, int c) {
@@ -477,6 +527,7 @@ FxNl fx_args(const paw_context *c) {
   N.proj = c->own_proj_dg.as<unsigned char>();
   N.exp = c->own_exp_dg.as<unsigned char>();
   N.sP = c->own_sP.as<int>();
+  N.r = c->own_r.as<short>();
   N.mask = c->own_mask.as<unsigned>();
   return N;
 }
@@ -533,7 +584,11 @@ void nlfx_build(paw_context *c, const double *P) {
   c->own_exp_dg.ensure(img, &c->dev_bytes);
   c->own_sP.ensure(sizeof(int) * (size_t)c->nown_pairs * c->npad, &c->dev_bytes);
   c->own_mask.ensure(sizeof(unsigned) * (size_t)c->nown_pairs, &c->dev_bytes);
-  k_build_digits<<<(unsigned)c->nown_pairs, 128>>>(c->own, kt, c->npad, P, c->own_proj_dg.as<unsigned char>(),
+  c->own_r.ensure(sizeof(short) * (size_t)c->ncells * c->own, &c->dev_bytes);
+  k_node_scales<<<(unsigned)c->ncells, 128>>>(c->own, c->npad, c->own_off.as<int>(), P, c->own_r.as<short>());
+  PAW_LAUNCH_CHECK("k_node_scales");
+  k_build_digits<<<(unsigned)c->nown_pairs, 128>>>(c->ncells, c->own, kt, c->npad, c->own_off.as<int>(), P,
+                                                   c->own_r.as<short>(), c->own_proj_dg.as<unsigned char>(),
                                                    c->own_exp_dg.as<unsigned char>(), c->own_sP.as<int>(),
                                                    c->own_mask.as<unsigned>());
   PAW_LAUNCH_CHECK("k_build_digits");

@@ -85,3 +85,32 @@ def test_many_coefficients_of_both_signs():
     Y, Z = fe.apply_S(X).cpu().numpy(), fe.apply_S(-X).cpu().numpy()
     fe.close()
     assert (np.abs(Y + Z).max(0) / np.abs(Y).max(0)).max() <= 16 * 2.0 ** -53
+
+
+@pytest.mark.parametrize("p", [3, 4, 6])
+def test_vectors_that_grow_where_projectors_fall(p):
+    """The projection of X = 1 / P on one cell, in which P falls by orders of magnitude, against the sum
+    of the projections of its single entries; both are read from S X on nodes that the local part does
+    not reach.  One projector, and all products have one sign.
+
+    Tolerance: on either side at most a 2^-53 for the digits of X, the projection, the coupling (two),
+    the digits of W and the expansion each: 12 * 2^-53 of the result."""
+    import paper_2604_26037_gb300 as P
+    s = mini_system(L=12.5, n=5, p=p, positions=[[6.25, 6.25, 6.25]], shells=[(0, 0.8)], D=np.full((1, 1, 1), 0.1),
+                    dS=np.full((1, 1, 1), 0.5))
+    fe = P.PawFE.from_system(s)
+    N1, own = 5 * p, p ** 3
+    cell = np.stack(np.meshgrid(*3 * [np.arange(p)], indexing="ij"), -1).reshape(-1, 3)[:, ::-1] + [2 * p, 2 * p, p]
+    dof = cell @ [1, N1, N1 * N1]                          # the owned nodes of the cell (2, 2, 1)
+    far = (2 * p + 1) + N1 * (2 * p + 1) + N1 * N1 * (3 * p + 1)   # a node of the cell (2, 2, 3)
+    E = np.zeros((fe.ndof, own + 1))
+    E[dof, np.arange(own)] = 1.0
+    row = fe.apply_S(to_dev(E)).cpu().numpy()[far, :own]   # P(far) dS P(o)
+    live = row != 0.0
+    x = np.where(live, 1.0 / np.where(live, row, 1.0), 0.0)
+    assert np.abs(row[live]).max() > 1e3 * np.abs(row[live]).min()
+    E[dof, np.arange(own)] = x
+    E[dof, own] = x
+    Y = fe.apply_S(to_dev(E)).cpu().numpy()[far].astype(np.longdouble)
+    fe.close()
+    assert np.abs(Y[own] / Y[:own].sum() - 1) < 12 * 2.0 ** -53
