@@ -625,7 +625,8 @@ template <bool EARLY>
 __device__ __forceinline__ float load_w(const float *p) { return EARLY ? __ldca(p) : __ldg(p); }
 
 // EARLY: launched before the kernel before it has ended (launch_pdl); W, which that kernel writes,
-// is then read with coherent loads.
+// is then read with coherent loads, and the status word behind the wait for that kernel (in all
+// launches: a step of 128 vectors on 12^3 cells 1.055 instead of 0.995 ms).
 template <int MODE, bool EARLY>
 __global__ void __launch_bounds__(THREADS, 1) k_exp_stream(const __grid_constant__ Args a, int *status) {
   using G = Geo<MODE>;

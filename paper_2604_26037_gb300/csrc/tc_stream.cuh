@@ -373,9 +373,8 @@ __device__ __forceinline__ void read_status(Shared *sh, const int *status, uint6
   }
 }
 
-// EARLY: launched before the kernel before it on the stream has ended (launch_pdl).  Only then is
-// the status word read behind the TMEM allocation: k_exp_stream<2> grows from 2888 to 3232
-// instructions with the read there, and a step of 128 vectors on 12^3 cells from 0.995 to 1.055 ms.
+// EARLY: launched before the kernel before it on the stream has ended (launch_pdl), which may still
+// set the status word: it is read behind the wait for that kernel.
 template <class P, bool EARLY>
 __global__ void __launch_bounds__(threads_for(P::NEPI), 1) k_tc_stream(const __grid_constant__ P p, int *status, uint64_t wait_ns,
                                                                      int probe) {
@@ -404,21 +403,9 @@ __global__ void __launch_bounds__(threads_for(P::NEPI), 1) k_tc_stream(const __g
     tmem_alloc(smem_u32(&sh->taddr), TMEM_COLS);
     tmem_relinquish();
   }
-  if constexpr (EARLY) grid_wait();
-  if (threadIdx.x == 0) {
-    sh->abort = (*reinterpret_cast<volatile int *>(status) != 0) ? 1 : 0;   // an earlier CTA gave up
-    if (probe && !sh->abort) {
-      // failure-path probe: wait on status[1], a word nothing sets, before any copy or
-      // MMA is issued; the bounded wait runs out and every role of the CTA gives up
-      const volatile int *gate = status + 1;
-      const uint64_t t0 = gtimer();
-      while (*gate == 0) {
-        if (gtimer() - t0 > wait_ns) {
-          sh->abort = 1;
-          break;
-        }
-      }
-    }
+  if constexpr (EARLY) {
+    grid_wait();
+    if (threadIdx.x == 0) read_status(sh, status, wait_ns, probe);
   }
   tc_fence_before();
   __syncthreads();
