@@ -392,6 +392,13 @@ struct PaddedIssue {
   ~PaddedIssue() { c->padded = PAD_NONE; }
 };
 
+// The sums U that an expansion of the loop cleared are clean for the loop's own next projection only
+struct CleanSums {
+  paw_context *c;
+  explicit CleanSums(paw_context *ctx) : c(ctx) { c->u_clean = 0; }
+  ~CleanSums() { c->u_clean = 0; }
+};
+
 static void block_step2(paw_context *c, const double *X, int ldx, int nb, int nbp, const ChebScalars &S, const double *hd,
                         const float *hf, int par, cudaStream_t s, const double *hd_dev, const float *hf_dev) {
   c->ws_lamp[par].ensure(sizeof(double) * S.nd, &c->dev_bytes);
@@ -414,7 +421,7 @@ static void block_step2(paw_context *c, const double *X, int ldx, int nb, int nb
 template <typename TR>
 static void block_loop(paw_context *c, paw_precision prec, const double *X, int ldx, int nout, int nb, double a0,
                        double cc, const ChebScalars &S, int par, double *Xo, int ldo, cudaStream_t s) {
-  c->u_clean = 0;
+  const CleanSums sums(c);
   const PaddedIssue padded(c, nb != nout ? PAD_SAME : PAD_NONE);   // nb columns are worked on, nout belong to the block
   const int64_t M = c->ndof;
   const int nsteps = S.nsteps;
@@ -499,7 +506,6 @@ static void block_loop(paw_context *c, paw_precision prec, const double *X, int 
   {
     PhaseScope ps(c, 5, s);
     op_Sinv<TR>(c, prec, RY, ldr, T, ldr, nb, s);
-    c->u_clean = 0;
     k_cheb_recover<TR><<<ew_grid(M, nout), blk, 0, s>>>(M, nout, T, ldr, X, ldx, d_lyfin, Xo, ldo);
     PAW_LAUNCH_CHECK("k_cheb_recover");
   }

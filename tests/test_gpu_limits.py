@@ -8,7 +8,8 @@ import time
 import numpy as np
 import pytest
 
-from tests.gpu_util import gpu_fe, to_dev
+from tests.gpu_util import gpu_fe, rel_err, to_dev
+from tests.oracle_systems import mini_system, sym_random
 
 pytestmark = pytest.mark.gpu
 
@@ -27,3 +28,50 @@ def test_probe_waits_one_limit():
     t = time.perf_counter() - t
     fe.close()
     assert 0.4 <= t < 0.6
+
+
+def _fill(leave):
+    """All device memory but about `leave` bytes."""
+    import torch
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    n = torch.cuda.mem_get_info()[0] - leave
+    for k in range(8):
+        try:
+            return torch.empty(n - (k << 21), dtype=torch.uint8, device="cuda")
+        except torch.OutOfMemoryError:
+            pass
+    pytest.skip("device memory could not be taken")
+
+
+def _one_atom(n, p):
+    import paper_2604_26037_gb300 as P
+    s = mini_system(L=2.5 * n, n=n, p=p, positions=[[2.2, 3.1, 4.4]], shells=[(0, 0.6), (1, 0.7)],
+                    D=sym_random(np.random.default_rng(3), 1, 4, 0.1), dS=sym_random(np.random.default_rng(4), 1, 4, 0.02))
+    return P.PawFE.from_system(s, block=16)
+
+
+def test_projection_sums_after_a_filter_that_failed():
+    """The first TF32 filter call fails between an expansion, which clears the projection sums for the
+    next step, and that step; an FP64 call then writes them.  A TF32 call has to clear them itself.
+    Tolerance: the TF32 rounding of the correction, as tests/test_gpu_ragged.py (1e-4)."""
+    import torch
+    from paper_2604_26037_gb300 import PawError
+    fe = _one_atom(6, 6)
+    X = to_dev(np.random.default_rng(2).standard_normal((fe.ndof, 16)))
+    Xf, Yf, Y = X.float(), torch.empty_like(X, dtype=torch.float32), torch.empty_like(X)
+    lam, bounds, out = np.linspace(0.1, 0.5, 16), (0.0, 0.6, 80.0), torch.empty_like(X)
+    ref = fe.apply_Sinv_approx(X).cpu().numpy()
+    fe.apply_Sinv_approx(Xf, prec="tf32")
+    fe.cheb_filter(X, lam, 4, bounds, prec="fp32", out=out)
+    hold = _fill(48 << 20)
+    try:
+        with pytest.raises(PawError, match="NO_MEMORY"):
+            fe.cheb_filter(X, lam, 4, bounds, prec="tf32", out=out)
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+    fe.apply_H(1e3 * X, Y=Y)
+    fe.apply_Sinv_approx(Xf, Y=Yf, prec="tf32")
+    assert rel_err(Yf.cpu().numpy(), ref) < 1e-4
+    fe.close()
