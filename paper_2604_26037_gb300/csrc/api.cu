@@ -918,6 +918,21 @@ static void copy_rows(const float *src, int lds, int n, float *dst, int ldd, int
   PAW_LAUNCH_CHECK("k_copy_rows");
 }
 
+// room for the padded copies of a block; where there is none the call goes without them
+static bool copies_fit(paw_context *c, size_t bytes) {
+  try {
+    c->ws_cx.ensure(bytes, &c->dev_bytes);
+    c->ws_cy.ensure(bytes, &c->dev_bytes);
+    return true;
+  } catch (const Error &e) {
+    if (e.code != PAW_ERR_NO_MEMORY) throw;
+    cudaGetLastError();
+    c->ws_cx.release(&c->dev_bytes);
+    c->ws_cy.release(&c->dev_bytes);
+    return false;
+  }
+}
+
 static void apply_any(paw_context *c, paw_precision prec, int which, const void *X, int ldx, void *Y, int ldy,
                       int ncols, cudaStream_t s) {
   if (prec == PAW_F32X2) {
@@ -932,15 +947,13 @@ static void apply_any(paw_context *c, paw_precision prec, int which, const void 
     return;
   }
   const bool rows16 = ncols % 4 == 0 && ldx % 4 == 0 && ldy % 4 == 0 && ((uintptr_t)X | (uintptr_t)Y) % 16 == 0;
+  const int np = std::min((ncols + 3) / 4 * 4, 512);
   if ((prec == PAW_TF32 || prec == PAW_BF16) && which != 1 && !rows16 && c->nown_pairs > 0 &&
-      c->tc_variant == 0) {
+      c->tc_variant == 0 && copies_fit(c, sizeof(float) * (size_t)c->ndof * np)) {
     // rows that are not whole 16-byte pieces: through zero-padded copies, on which the persistent
     // tensor-core kernels run (approximate inverse overlap, degree 6, 12^3 cells, 130 columns: 0.67
     // instead of 1.03 ms; H 1.14 instead of 1.69 ms; no slower on 4^3 cells of degree 4)
     // in blocks of at most 512 columns, which bounds the copies
-    const int np = std::min((ncols + 3) / 4 * 4, 512);
-    c->ws_cx.ensure(sizeof(float) * (size_t)c->ndof * np, &c->dev_bytes);
-    c->ws_cy.ensure(sizeof(float) * (size_t)c->ndof * np, &c->dev_bytes);
     float *xs = c->ws_cx.as<float>(), *ys = c->ws_cy.as<float>();
     const PaddedIssue padded(c, PAD_CELL);
     for (int j = 0; j < ncols; j += np) {

@@ -75,3 +75,22 @@ def test_projection_sums_after_a_filter_that_failed():
     fe.apply_Sinv_approx(Xf, Y=Yf, prec="tf32")
     assert rel_err(Yf.cpu().numpy(), ref) < 1e-4
     fe.close()
+
+
+def test_ragged_blocks_without_room_for_copies():
+    """130 columns of 36^3 nodes, whose padded copies (25 MB each) do not fit: the call goes without them."""
+    import torch
+    fe = _one_atom(6, 6)
+    X = to_dev(np.random.default_rng(3).standard_normal((fe.ndof, 130)))
+    Xf, Yf = X.float(), torch.empty_like(X, dtype=torch.float32)
+    ref = fe.apply_Sinv_approx(X).cpu().numpy()
+    whole = Xf[:, :128].contiguous()
+    fe.apply_Sinv_approx(whole, prec="tf32")               # the images of the projectors
+    hold = _fill(20 << 20)
+    try:
+        fe.apply_Sinv_approx(Xf, Y=Yf, prec="tf32")
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+    assert rel_err(Yf.cpu().numpy(), ref) < 1e-4
+    fe.close()
