@@ -926,7 +926,6 @@ static bool copies_fit(paw_context *c, size_t bytes) {
     return true;
   } catch (const Error &e) {
     if (e.code != PAW_ERR_NO_MEMORY) throw;
-    cudaGetLastError();
     c->ws_cx.release(&c->dev_bytes);
     c->ws_cy.release(&c->dev_bytes);
     return false;

@@ -38,6 +38,7 @@ paw_status fail(paw_status code, const std::string &msg);
   do {                                                                        \
     cudaError_t e_ = (call);                                                  \
     if (e_ != cudaSuccess) {                                                  \
+      cudaGetLastError();   /* reported here, not by a later launch check */  \
       throw ::pawfe::Error{e_ == cudaErrorMemoryAllocation ? PAW_ERR_NO_MEMORY \
                                                            : PAW_ERR_CUDA,     \
                            std::string(#call) + ": " + cudaGetErrorString(e_)}; \

@@ -51,6 +51,29 @@ def _one_atom(n, p):
     return P.PawFE.from_system(s, block=16)
 
 
+def test_a_failed_allocation_ends_with_its_call():
+    """The cell matrices of the first TF32 product (107 MB) do not fit; what the caller launches next, and
+    the FP64 call after it, work.  Tolerance: the FP64 sums of a node in another order."""
+    import torch
+    from paper_2604_26037_gb300 import PawError
+    fe = _one_atom(6, 6)
+    X = to_dev(np.random.default_rng(1).standard_normal((fe.ndof, 16)))
+    Xf, Yf, Y = X.float(), torch.empty_like(X, dtype=torch.float32), torch.empty_like(X)
+    ref = fe.apply_H(X).cpu().numpy()
+    fe.apply_Sinv_approx(Xf, prec="tf32")
+    hold = _fill(48 << 20)
+    try:
+        with pytest.raises(PawError, match="NO_MEMORY"):
+            fe.apply_H(Xf, Y=Yf, prec="tf32")
+        X.mul_(2.0)
+        fe.apply_H(X, Y=Y)
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+    assert rel_err(Y.cpu().numpy(), 2.0 * ref) < 1e-13
+    fe.close()
+
+
 def test_projection_sums_after_a_filter_that_failed():
     """The first TF32 filter call fails between an expansion, which clears the projection sums for the
     next step, and that step; an FP64 call then writes them.  A TF32 call has to clear them itself.
