@@ -357,6 +357,12 @@ paw_status paw_batch_cheb_filter(paw_batch b, paw_precision prec, const paw_batc
         }
         b->sig = sig;
       }
+      // images of a potential that changed since the capture (their launches are not in the graph)
+      for (size_t i = 0; i < n; ++i) {
+        if (!plan[i].valid) continue;
+        local_prepare(b->inst[i], s);
+        if (prec == PAW_TF32 || prec == PAW_BF16) tc_prepare(b->inst[i], prec, s);
+      }
       PAW_CUDA(cudaGraphLaunch(b->exec, s));
       PAW_CUDA(cudaStreamSynchronize(s));
     }

@@ -355,6 +355,8 @@ void nlfx_project(paw_context *c, const double *X, int ldx, int ncols, const dou
 void nlfx_expand(paw_context *c, int mode, const ExpArgs &A, const double *W1, const double *W2, cudaStream_t s);
 // sum-factorised local operator on FP64 data (sumfac.cu):
 // Y += alpha * (cK K^e + cV V^e + (cM + cMcol[j]) M^e) X, cell by cell with assembly;
+// (local_prepare: its image of the potential, made again after a change)
+void local_prepare(paw_context *c, cudaStream_t s);
 void local_sf(paw_context *c, const double *X, int ldx, double *Y, int ldy, int ncols, double alpha,
               double cK, double cV, double cM, const double *cMcol, cudaStream_t s);
 // out[e][q] = wq[q] sum_v f[v] u_v(x_q)^2 at the (p+2)^3 Gauss points of every cell (wq, f NULL: 1)

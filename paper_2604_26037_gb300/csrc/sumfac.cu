@@ -922,18 +922,20 @@ template void density_sf<double>(paw_context *, const double *, int, int, const 
 template void density_sf<float>(paw_context *, const float *, int, int, const double *, const double *, double *,
                                 cudaStream_t);
 
+void local_prepare(paw_context *c, cudaStream_t s) {
+  if (c->Vfx_valid) return;
+  c->Vfx.ensure(sizeof(fx2) * (size_t)c->ncells * c->nq, &c->dev_bytes);
+  c->Vfx_exp.ensure(sizeof(int) * (size_t)c->ncells, &c->dev_bytes);
+  k_V_fx<<<(unsigned)c->ncells, 128, 0, s>>>(c->nq, c->Vq.as<double>(), c->Vfx.as<fx2>(), c->Vfx_exp.as<int>());
+  PAW_LAUNCH_CHECK("k_V_fx");
+  c->Vfx_valid = 1;
+}
+
 void local_sf(paw_context *c, const double *X, int ldx, double *Y, int ldy, int ncols, double alpha, double cK,
               double cV, double cM, const double *cMcol, cudaStream_t s) {
   if (ncols <= 0) return;
   FxLocal t = plans(c).local_tables(c, alpha, cK, cV, cM);
-  // V_q per cell (rebuilt lazily after a potential change)
-  if (!c->Vfx_valid) {
-    c->Vfx.ensure(sizeof(fx2) * (size_t)c->ncells * c->nq, &c->dev_bytes);
-    c->Vfx_exp.ensure(sizeof(int) * (size_t)c->ncells, &c->dev_bytes);
-    k_V_fx<<<(unsigned)c->ncells, 128, 0, s>>>(c->nq, c->Vq.as<double>(), c->Vfx.as<fx2>(), c->Vfx_exp.as<int>());
-    PAW_LAUNCH_CHECK("k_V_fx");
-    c->Vfx_valid = 1;
-  }
+  local_prepare(c, s);
   t.cell_dofs = c->cell_dofs.as<int>();
   t.V = c->Vfx.as<fx2>();
   t.sV = c->Vfx_exp.as<int>();
