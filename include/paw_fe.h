@@ -289,8 +289,9 @@ paw_status paw_cheb_filter(paw_handle h, paw_precision prec, const double *X_in,
  * instance is captured once into a single CUDA graph: instances run on up to
  * `streams` concurrent branches of the graph, and each call replays the whole
  * batch with one cudaGraphLaunch.  The graph is recaptured when a problem's
- * pointers, sizes, degree, bounds or the precision change; eigenvalue
- * estimates (lambda_in) may change freely between calls.
+ * pointers, sizes, degree, bounds or the precision change, and when other calls
+ * on a handle have replaced the workspaces that it uses; eigenvalue
+ * estimates (lambda_in), the potential and D_ij may change freely between calls.
  *
  * Autotuning (options.autotune = 1) happens on the first call and after a
  * recapture: for every instance the tensor-core kernel family (persistent

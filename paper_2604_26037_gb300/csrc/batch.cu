@@ -45,6 +45,7 @@ struct paw_batch_s {
   int captures = 0;
   int branches = 1;
   std::vector<double> sig;               // signature of the captured graph
+  std::vector<const void *> held;        // buffers of the instances that it holds by address
   double *hd = nullptr;                  // pinned scalar images
   float *hf = nullptr;
   size_t hd_cap = 0, hf_cap = 0;
@@ -99,6 +100,24 @@ void issue_instance(paw_batch_s *b, paw_precision prec, const paw_batch_problem 
     pawfe::cheb_issue(c, prec, q.X_in + j0, q.ldx, nb, nb, q.bounds, P.blocks[k], b->hd + P.hd_off[k],
                       b->hf + P.hf_off[k], q.X_out + j0, q.ldo, s);
   }
+}
+
+// Buffers of the instances that grow on use and that captured launches hold by address (0: not made
+// yet): a call on a handle between two batched calls may have replaced them.
+std::vector<const void *> held_buffers(const paw_batch_s *b) {
+  std::vector<const void *> v;
+  for (const paw_context *c : b->inst)
+    for (const pawfe::DevBuf *d :
+         {&c->ws_lamp[0], &c->ws_cfp[0], &c->ws_Y0p[0], &c->ws_RX, &c->ws_RY, &c->ws_T, &c->ws_Y0f, &c->ws_Y0lo, &c->ws_W,
+          &c->scr_main.partial, &c->scr_main.pp, &c->scr_main.W2, &c->Vfx, &c->Vfx_exp, &c->tc_tf32.He, &c->tc_bf16.He})
+      v.push_back(d->ptr);
+  return v;
+}
+bool still_held(const paw_batch_s *b) {
+  const std::vector<const void *> now = held_buffers(b);
+  for (size_t i = 0; i < b->held.size(); ++i)
+    if (b->held[i] && b->held[i] != now[i]) return false;
+  return true;
 }
 
 // Capture every valid instance into one graph with `branches` concurrent
@@ -306,7 +325,7 @@ paw_status paw_batch_cheb_filter(paw_batch b, paw_precision prec, const paw_batc
                           q.bounds.bW, q.bounds.bU, (double)(uintptr_t)q.X_out, (double)q.ldo};
       sig.insert(sig.end(), v, v + 9);
     }
-    bool rebuild = b->exec == nullptr || sig != b->sig;
+    bool rebuild = b->exec == nullptr || sig != b->sig || !still_held(b);
     if (nd > b->hd_cap || nf > b->hf_cap) {   // captured copies read the arenas: new arenas, new graph
       PAW_CUDA(cudaStreamSynchronize(s));
       if (b->hd) cudaFreeHost(b->hd);
@@ -356,6 +375,7 @@ paw_status paw_batch_cheb_filter(paw_batch b, paw_precision prec, const paw_batc
           capture(b, prec, problems, plan, maxbr);
         }
         b->sig = sig;
+        b->held = held_buffers(b);
       }
       // images of a potential that changed since the capture (their launches are not in the graph)
       for (size_t i = 0; i < n; ++i) {

@@ -38,3 +38,29 @@ def test_replay_after_a_change_of_the_potential(prec):
         batch.close()
         for fe in fes:
             fe.close()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "tf32"])
+def test_replay_after_the_workspaces_have_grown(prec):
+    """Wider calls on the handles give them larger workspaces: the graph is captured again."""
+    import torch
+    import paper_2604_26037_gb300 as P
+    systems, fes, probs = _instances()
+    probs = [[X[:, :8].contiguous(), lam[:8], m, bd] for X, lam, m, bd in probs]
+    batch = P.PawBatch(fes, streams=2, autotune=False)
+    try:
+        st, outs = _run_batch(batch, probs, prec)
+        captures = batch.tuning(0)["captures"]
+        for fe, (X, lam, m, bd) in zip(fes, probs):
+            fe.apply_H(torch.randn(fe.ndof, 200, dtype=torch.float64, device="cuda"))
+            fe.cheb_filter(torch.cat([X, X], 1), [*lam, *lam], m, bd, prec=prec)
+        for out in outs:
+            out.zero_()
+        st, outs = _run_batch(batch, probs, prec, outs=outs)
+        assert st == [0] * len(fes) and batch.tuning(0)["captures"] == captures + 1
+        for fe, (X, lam, m, bd), out in zip(fes, probs, outs):
+            assert rel_err(out.cpu().numpy(), fe.cheb_filter(X, lam, m, bd, prec=prec).cpu().numpy()) < TOL[prec]
+    finally:
+        batch.close()
+        for fe in fes:
+            fe.close()
