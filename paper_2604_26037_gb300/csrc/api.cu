@@ -1182,6 +1182,7 @@ paw_status paw_get_info(paw_handle c, paw_info *out) {
 paw_status paw_set_veff(paw_handle c, const double *V_q) {
   PAW_TRY_BEGIN
   PAW_REQUIRE(c && V_q, PAW_ERR_INVALID_ARG, "NULL handle or V_q");
+  PAW_CUDA(cudaDeviceSynchronize());   // calls in flight keep the potential that they were issued with
   PAW_CUDA(cudaMemcpy(c->Vq.ptr, V_q, sizeof(double) * (size_t)c->ncells * c->nq, cudaMemcpyDeviceToDevice));
   rebuild_hamiltonian(c);
   return PAW_OK;

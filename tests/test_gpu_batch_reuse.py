@@ -1,4 +1,5 @@
-"""GPU: a batch whose handles are used by other calls between its replays.
+"""GPU: a batch whose handles are used by other calls between its replays, and a potential that is set
+behind a call in flight.
 
 Tolerances and instances: tests/test_gpu_batch.py.
 """
@@ -64,3 +65,28 @@ def test_replay_after_the_workspaces_have_grown(prec):
         batch.close()
         for fe in fes:
             fe.close()
+
+
+def test_potential_set_behind_a_filter_on_another_stream():
+    """set_veff takes no stream: a filter call in flight on a stream of the caller's keeps the potential
+    that it was issued with (FP64; 64 vectors of 24^3 nodes, 30 steps)."""
+    import torch
+    import paper_2604_26037_gb300 as P
+    from tests.oracle_systems import mini_system, sym_random
+    rng = np.random.default_rng(5)
+    s = mini_system(L=15.0, n=6, p=4, positions=[[2.2, 3.1, 4.4], [8.1, 7.7, 6.2]], shells=[(0, 0.6), (1, 0.7)],
+                    D=sym_random(rng, 2, 4, 0.1), dS=sym_random(rng, 2, 4, 0.02))
+    fe = P.PawFE.from_system(s, block=64)
+    X, out = torch.randn(fe.ndof, 64, dtype=torch.float64, device="cuda"), torch.empty(fe.ndof, 64, dtype=torch.float64,
+                                                                                   device="cuda")
+    V = [torch.full((216, 216), v, dtype=torch.float64, device="cuda") for v in (0.0, 1.0)]
+    args = (np.linspace(0.1, 0.5, 64), 30, (0.0, 0.6, 60.0))
+    fe.set_veff(V[0])
+    ref = fe.cheb_filter(X, *args, prec="fp64").cpu().numpy()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(torch.cuda.Stream()):
+        fe.cheb_filter(X, *args, prec="fp64", out=out)
+    fe.set_veff(V[1])
+    torch.cuda.synchronize()
+    assert rel_err(out.cpu().numpy(), ref) < 1e-11
+    fe.close()
