@@ -419,30 +419,6 @@ def run_ours(args, ws, rank, local):
         fp64 = {"value": whole_job_rate(units_per_step, ws, ms64), "ms_per_step": ms64,
                 "steps": args.fp64_steps, "warmup": 1}
 
-    # the same filter with options.y0_pair32 (served by the FP64 kernels of step 2)
-    pair = None
-    if args.pair_steps > 0 and not kp and not args.y0_pair32:
-        fe_p = P.PawFE.from_system(sysd, block=cfg["block"], y0_fp32=args.y0_fp32, y0_pair32=True,
-                                   overlap=not args.no_overlap)
-        out_p = torch.empty_like(out)
-        ms_p, prof_p, clk_p = timed(args.prec, args.pair_steps, 1, profile=True, h=fe_p, dst=out_p)
-        # both handles filter the same input with the FP64 bracket: the outputs differ
-        # by the step-2 rounding only
-        fe.cheb_filter(X, lam, m, bounds, prec="fp64", out=out)
-        fe_p.cheb_filter(X, lam, m, bounds, prec="fp64", out=out_p)
-        diff64 = float((out_p - out).abs().max() / out.abs().max())
-        ph = {k: round(v["ms"] / args.pair_steps, 3) for k, v in prof_p.items() if isinstance(v, dict)}
-        ph64 = {k: v["ms"] / args.steps for k, v in prof.items() if isinstance(v, dict)}
-        s2 = ph["residual_local"] + ph["residual_nonlocal"]
-        s2_64 = ph64["residual_local"] + ph64["residual_nonlocal"]
-        pair = {"value": round(whole_job_rate(units_per_step, ws, ms_p), 4), "ms_per_step": round(ms_p, 3),
-                "steps": args.pair_steps, "warmup": 1, "phases_ms_per_step": ph,
-                "step2_ms": round(s2, 3), "step2_speedup_vs_fp64": round(s2_64 / s2, 3),
-                "fp64_bracket_output_rel_diff": diff64, "clocks": clk_p,
-                "arithmetic": "options.y0_pair32: step 2 by the same FP64-accurate kernels as without it"}
-        del out_p
-        fe_p.close()
-
     # end to end through the public API with host buffers (pinned), copies inside the timed
     # region: every step copies the whole block in, filters it with one call and copies the
     # result out.  Consecutive steps are pipelined with three device buffer sets: the input of
@@ -655,8 +631,6 @@ def run_ours(args, ws, rank, local):
     }
     if acc is not None:
         res["accuracy"] = acc
-    if pair is not None:
-        res["step2_pair32"] = pair
     if rrm is not None:
         res["rayleigh_ritz"] = rrm
     if gradm is not None:
@@ -724,7 +698,7 @@ def sf_flops_per_cell_vec(n1):
     fl += lines * (2 * split(n1) + 3 * 2 * eo(n1, n1) + 2 * n1 + 2 * outs(n1))  # S, R (R = kf T + c S on the halves)
     fl += n1 * n1 * (split(n1) + 2 * eo(q1, n1) + outs(q1))                      # U1
     fl += q1 * n1 * (split(n1) + 2 * eo(q1, n1) + outs(q1))                      # U2
-    fl += q1 * q1 * (split(n1) + 2 * eo(q1, n1) + outs(q1) + q1)                 # U3 (times w V)
+    fl += q1 * q1 * (split(n1) + 2 * eo(q1, n1) + outs(q1) + q1)                 # U3 (times V)
     fl += q1 * q1 * (split(q1) + 2 * eo(n1, q1) + outs(n1))                      # B2
     fl += q1 * n1 * (split(q1) + 2 * eo(n1, q1) + outs(n1))                      # B1
     # y: the last kinetic / mass and potential contractions in one accumulator per line
@@ -956,9 +930,7 @@ def main():
                     help="R-ChFSI iterations of the accuracy leg, mixed vs FP64 filter (0: skip)")
     ap.add_argument("--y0-fp32", action="store_true")
     ap.add_argument("--y0-pair32", action="store_true",
-                    help="set options.y0_pair32 in the main measurement")
-    ap.add_argument("--pair-steps", type=int, default=3,
-                    help="timed calls of the filter with options.y0_pair32, reported beside the main one (0: skip)")
+                    help="set options.y0_pair32 (step 2 by the same kernels, FP64 accuracy)")
     ap.add_argument("--no-e2e", action="store_true")
     ap.add_argument("--no-overlap", action="store_true",
                     help="filter the blocks one after another (no overlap of step 2 with the previous block's loop)")
