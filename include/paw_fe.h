@@ -84,9 +84,14 @@ typedef enum {
 
 typedef enum {
   PAW_FP64 = 0,  /* FP64 data and FP64-level accuracy in every step: the plain */
-                 /* method (the cell and projector contractions run in 55- to  */
-                 /* 59-bit fixed point per cell and vector, with errors no     */
-                 /* larger than those of FP64 sums)                            */
+                 /* method.  The cell and projector contractions run in 54- to */
+                 /* 59-bit fixed point with one scale per cell and vector (and */
+                 /* one per row of the tables).  Relative to the sum of the    */
+                 /* magnitudes of its terms an entry has about the error of an */
+                 /* FP64 sum (local part: 0.5 to 1.3 of it, up to 5 in cells   */
+                 /* that a potential of 30 Ha dominates); an entry whose terms */
+                 /* are all far below the largest of its cell and vector keeps */
+                 /* an error of 2^-54 of that largest one                      */
   PAW_FP32 = 1,  /* filter bracket in FP32 storage and FP32 FMA arithmetic     */
   PAW_TF32 = 2,  /* FP32 storage; cell products and projector contractions   */
                  /* on tcgen05 tensor cores (TF32 operands, FP32 accumulation */

@@ -231,9 +231,9 @@ __device__ __forceinline__ int fx_gather(const int *cell_dofs, const T *X, int64
 }
 
 // What bounds it: the IMAD pipe, three IMAD.WIDE per product at 32 per clock and SM (measured;
-// some 40% of all instructions at p = 6): 6.8 ms of the 9.5 ms per 256 vectors of 16^3 cells at
-// p = 6 (9.9 ms with the sums of the accumulator pairs on that pipe too), the rest barriers and
-// dependent issue.  The same contractions
+// some 40% of all instructions at p = 6): 6.8 ms of the 9.7 ms per 256 vectors of 16^3 cells at
+// p = 6 (9.5 ms without the row scales; 9.9 ms with the sums of the accumulator pairs on that pipe
+// too), the rest barriers and dependent issue.  The same contractions
 // with FP64 FMAs took 53.2 ms there (FP64 pipe 88% busy); p = 4: 2.9 ms.
 // The tables are kernel parameters, read by the IMADs as constant operands.  The nodal tensor
 // of the potential part grows in place to the (p+2)^3 Gauss points and back (W); the kinetic
