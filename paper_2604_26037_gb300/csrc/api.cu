@@ -1137,7 +1137,7 @@ paw_status paw_destroy(paw_handle c) {
   cudaDeviceSynchronize();
   DevBuf *bufs[] = {&c->cell_dofs, &c->md_inv64, &c->md_inv32, &c->He64, &c->He32, &c->Me64, &c->Me32,
                     &c->K64, &c->Nq64, &c->wq64, &c->Vq, &c->tc_tf32.He, &c->tc_tf32.Me, &c->tc_bf16.He,
-                    &c->tc_bf16.Me, &c->ent_dof, &c->P64, &c->P32, &c->own_off, &c->own_atom, &c->own_proj_dg, &c->own_exp_dg, &c->own_sP, &c->own_mask, &c->own_r,
+                    &c->tc_bf16.Me, &c->ent_dof, &c->P64, &c->P32, &c->own_off, &c->own_atom, &c->own_proj_dg, &c->own_exp_dg, &c->own_sP, &c->own_mask, &c->own_r, &c->own_P64,
                     &c->ownP32,
                     &c->DH64, &c->DS64, &c->DSinv64, &c->ws_W, &c->ws_RX,
                     &c->ws_RY, &c->ws_T, &c->ws_Y0f, &c->ws_colscale, &c->ws_red, &c->ws_vec,

@@ -216,6 +216,7 @@ struct paw_context {
   // expansion, exponent per pair and projector, node tiles with nonzero values per pair, row
   // exponents per cell and owned node (int16)
   pawfe::DevBuf own_proj_dg, own_exp_dg, own_sP, own_mask, own_r;
+  pawfe::DevBuf own_P64;                      // P of the pairs itself, for cells of one owned node
   int64_t proj_nnz = 0;                       // nonzero (owned node, projector) entries over all pairs
   pawfe::DevBuf apair_off, apair;             // atom-major list of the pairs (int32)
   // atom-pair Gram blocks G_ab = P^a^T M_D^-1 P^b for atoms with common support

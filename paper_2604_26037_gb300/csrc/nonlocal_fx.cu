@@ -24,6 +24,7 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 #include "fx64.cuh"
@@ -455,6 +456,67 @@ __global__ void __launch_bounds__(256, 2) k_fx_expand(FxNl N, ExpArgs A, const d
   }
 }
 
+// Cells of one owned node (degree 1) fill one of the 16 rows of a digit tile: FP64 FMAs over the
+// nonzero entries instead, lane = vector.  Bound by the per-pair partials (16 values written and read
+// again for one node) and, for few vectors, by the chain over the pairs of a cell, which four warps of the
+// expansion share.  On 24^3 cells with 216 atoms, 64 vectors: approximate inverse overlap 0.90
+// ms (digits 2.17), H 1.06 (2.26), a filter of 8 steps 11.1 (29.4).  For the eight nodes of degree 2
+// the digits are faster (16^3 cells, 64 vectors: H 0.82 ms, FMAs in this form 1.81).
+template <int NPAD, bool SCALED>
+__global__ void __launch_bounds__(256) k_one_project(FxNl A, const double *__restrict__ P, const double *__restrict__ X,
+                                                     int64_t ldx, int ncols, const double *__restrict__ rowscale,
+                                                     double *__restrict__ U) {
+  const int ntile = (ncols + 31) / 32;
+  const int e = blockIdx.x / ntile, v = (blockIdx.x - e * ntile) * 32 + (threadIdx.x & 31);
+  const int k0 = A.own_off[e], k1 = A.own_off[e + 1];
+  if (k0 == k1 || v >= ncols) return;
+  const int64_t d = owned_base(e, A.n, A.p, A.N1);
+  double x = X[d * ldx + v];
+  if (SCALED) x *= rowscale[d];
+  for (int u = threadIdx.x >> 5; u < (k1 - k0) * NPAD; u += 8) {
+    const double c = __ldg(P + (size_t)k0 * NPAD + u);
+    U[((size_t)k0 * NPAD + u) * ncols + v] = c != 0.0 ? c * x : 0.0;
+  }
+}
+
+template <int NPAD, int MODE>
+__global__ void __launch_bounds__(128) k_one_expand(FxNl N, ExpArgs A, const double *__restrict__ P,
+                                                    const double *__restrict__ W1, const double *__restrict__ W2) {
+  constexpr int NW = (MODE == EXP_RECURRENCE) ? 2 : 1;
+  __shared__ double part[NW][4][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, ncols = A.ncols, ntile = (ncols + 31) / 32;
+  const int e = blockIdx.x / ntile, v = (blockIdx.x - e * ntile) * 32 + lane, vc = min(v, ncols - 1);
+  double s[NW] = {};
+  for (int k = N.own_off[e] + warp; k < N.own_off[e + 1]; k += 4) {
+    const size_t w = (size_t)N.own_atom[k] * NPAD * ncols + vc;
+#pragma unroll
+    for (int al = 0; al < NPAD; ++al) {
+      const double c = __ldg(P + (size_t)k * NPAD + al);
+      if (c == 0.0) continue;
+#pragma unroll
+      for (int i = 0; i < NW; ++i) s[i] = fma(c, __ldg((i ? W2 : W1) + w + (size_t)al * ncols), s[i]);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < NW; ++i) part[i][warp][lane] = s[i];
+  __syncthreads();
+  if (warp || v >= ncols) return;
+#pragma unroll
+  for (int i = 0; i < NW; ++i) s[i] = (part[i][0][lane] + part[i][1][lane]) + (part[i][2][lane] + part[i][3][lane]);
+  const int64_t d = owned_base(e, N.n, N.p, N.N1);
+  double *Y = static_cast<double *>(A.Y) + d * A.ldy + v;
+  if (MODE == EXP_SET) {
+    *Y = s[0];
+    return;
+  }
+  const double x = static_cast<const double *>(A.Xin)[d * A.ldx + v];
+  *Y = static_cast<const double *>(A.mdinv)[d] * (x - s[0]);
+  if (MODE == EXP_RECURRENCE) {
+    double *RX = static_cast<double *>(A.RX) + d * A.ldx + v;
+    *RX = fma(A.c64[v], static_cast<const double *>(A.Y0)[d * A.ldy0 + v], -A.beta * x - A.gamma * *RX + s[NW - 1]);
+  }
+}
+
 // row exponents of one cell per block: that of the largest entry of the row over the cell's pairs
 __global__ void __launch_bounds__(128) k_node_scales(int own, int npad, const int *__restrict__ own_off,
                                                      const double *__restrict__ P, short *__restrict__ r) {
@@ -578,6 +640,12 @@ void expand_mode(paw_context *c, int mode, const ExpArgs &A, const double *W1, c
 
 void nlfx_build(paw_context *c, const double *P) {
   if (c->nown_pairs == 0) return;
+  if (c->own == 1) {
+    const size_t bytes = sizeof(double) * (size_t)c->nown_pairs * c->npad;
+    c->own_P64.ensure(bytes, &c->dev_bytes);
+    PAW_CUDA(cudaMemcpy(c->own_P64.ptr, P, bytes, cudaMemcpyDeviceToDevice));
+    return;
+  }
   const int kt = (c->own + 15) / 16, mt = c->npad / 16;
   const size_t img = (size_t)c->nown_pairs * kt * mt * DG * 256;
   c->own_proj_dg.ensure(img, &c->dev_bytes);
@@ -603,6 +671,18 @@ void nlfx_project(paw_context *c, const double *X, int ldx, int ncols, const dou
                   cudaStream_t s) {
   PAW_REQUIRE(c->own <= 512 && (c->npad == 16 || c->npad == 32), PAW_ERR_UNSUPPORTED,
               "projection tile exceeds shared memory (degree too high)");
+  if (c->own == 1) {
+    auto run = [&](auto kern) {
+      kern<<<(unsigned)((int64_t)c->ncells * ((ncols + 31) / 32)), 256, 0, s>>>(fx_args(c), c->own_P64.as<double>(), X, ldx,
+                                                                                ncols, rowscale, U);
+      PAW_LAUNCH_CHECK("k_one_project");
+    };
+    if (c->npad == 16)
+      rowscale ? run(k_one_project<16, true>) : run(k_one_project<16, false>);
+    else
+      rowscale ? run(k_one_project<32, true>) : run(k_one_project<32, false>);
+    return;
+  }
   const bool narrow = ncols <= 16 || (size_t)DG * (c->own + 15) * 64 > FX_SMEM_MAX;
   if (c->npad == 16)
     narrow ? launch_project<16, 16>(c, X, ldx, ncols, rowscale, U, s)
@@ -615,6 +695,21 @@ void nlfx_project(paw_context *c, const double *X, int ldx, int ncols, const dou
 void nlfx_expand(paw_context *c, int mode, const ExpArgs &A, const double *W1, const double *W2, cudaStream_t s) {
   PAW_REQUIRE(c->max_own_pairs <= PAIRS_PER_CELL_MAX && c->own <= 512, PAW_ERR_UNSUPPORTED,
               "too many atoms on one cell for the expansion kernel");
+  if (c->own == 1) {
+    auto run = [&](auto kern) {
+      kern<<<(unsigned)((int64_t)c->ncells * ((A.ncols + 31) / 32)), 128, 0, s>>>(fx_args(c), A, c->own_P64.as<double>(), W1,
+                                                                                  W2);
+      PAW_LAUNCH_CHECK("k_one_expand");
+    };
+    auto of = [&](auto np) {
+      constexpr int NPAD = decltype(np)::value;
+      mode == EXP_SET    ? run(k_one_expand<NPAD, EXP_SET>)
+      : mode == EXP_SINV ? run(k_one_expand<NPAD, EXP_SINV>)
+                         : run(k_one_expand<NPAD, EXP_RECURRENCE>);
+    };
+    c->npad == 16 ? of(std::integral_constant<int, 16>{}) : of(std::integral_constant<int, 32>{});
+    return;
+  }
   const bool narrow = A.ncols <= 16 || expand_smem(c, 32) > FX_SMEM_MAX;
   if (c->npad == 16)
     narrow ? expand_mode<16, 16>(c, mode, A, W1, W2, s) : expand_mode<16, 32>(c, mode, A, W1, W2, s);

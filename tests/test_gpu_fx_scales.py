@@ -114,3 +114,28 @@ def test_vectors_that_grow_where_projectors_fall(p):
     Y = fe.apply_S(to_dev(E)).cpu().numpy()[far].astype(np.longdouble)
     fe.close()
     assert np.abs(Y[own] / Y[:own].sum() - 1) < 12 * 2.0 ** -53
+
+
+@pytest.mark.parametrize("nproj", [4, 18])
+@pytest.mark.parametrize("ncols", [1, 32, 33])
+def test_one_owned_node_per_cell(nproj, ncols):
+    """Degree 1, whose projector contractions are FP64 FMAs: every output stage against the oracle, with
+    atoms on every cell and none, and values on nodes without projectors left out (FP64 tolerances of the
+    other degrees)."""
+    import paper_2604_26037_gb300 as P
+    from oracle import cheb
+    from oracle import ops as O
+    rng = np.random.default_rng(nproj + ncols)
+    shells = [(0, 0.5), (1, 0.45)] if nproj == 4 else [(0, 0.5), (0, 0.4), (1, 0.5), (1, 0.45), (2, 0.5), (2, 0.4)]
+    for n, na in ((6, 20), (9, 2)):
+        s = mini_system(L=1.5 * n, n=n, p=1, positions=rng.uniform(0.0, 1.5 * n, (na, 3)), shells=shells, vdepth=1.0,
+                        D=sym_random(rng, na, nproj, 0.1), dS=sym_random(rng, na, nproj, 0.005))
+        op, fe = O.PawOperators(s), P.PawFE.from_system(s, block=64)
+        X, lam, b = rng.standard_normal((op.mesh.ndof, ncols)), np.linspace(0.1, 0.9, ncols), (0.0, 1.0, 60.0)
+        Xd = to_dev(X)
+        assert rel_err(fe.apply_H(Xd).cpu().numpy(), op.apply_H(X)) < TOL
+        assert rel_err(fe.apply_S(Xd).cpu().numpy(), op.apply_S(X)) < TOL
+        assert rel_err(fe.apply_Sinv_approx(Xd).cpu().numpy(), op.apply_Sinv_approx(X)) < TOL
+        ref = cheb.rchfsi_filter(op.apply_H, op.apply_S, op.apply_Sinv_approx, X, lam, 4, *b)
+        assert rel_err(fe.cheb_filter(Xd, lam, 4, b, prec="fp64").cpu().numpy(), ref) < 1e-10
+        fe.close()
