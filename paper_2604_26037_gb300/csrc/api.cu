@@ -80,6 +80,12 @@ void encode_row_map(CUtensorMap *map, const float *base, int64_t rows, int cols,
   PAW_REQUIRE(r == CUDA_SUCCESS, PAW_ERR_CUDA, "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")");
 }
 
+void cuda_fail(cudaError_t e, const char *call) {
+  cudaGetLastError();
+  throw Error{e == cudaErrorMemoryAllocation ? PAW_ERR_NO_MEMORY : PAW_ERR_CUDA,
+              std::string(call) + ": " + cudaGetErrorString(e)};
+}
+
 void DevBuf::ensure(size_t nbytes, int64_t *counter) {
   if (nbytes <= bytes && ptr) return;
   if (ptr) {
