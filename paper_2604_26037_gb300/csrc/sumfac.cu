@@ -779,8 +779,8 @@ struct SfPlans {
     return t;
   }
   // largest |a| (A_b B_c) + |b| (B_b A_c) over two rows b, c: bound of a A (x) B + b B (x) A
-  static long double pair_bound(long double a, long double b, const Tab1 &A, const Tab1 &B) {
-    long double m = 0;
+  static double pair_bound(double a, double b, const Tab1 &A, const Tab1 &B) {
+    double m = 0.0;
     for (size_t i = 0; i < A.row.size(); ++i)
       for (size_t j = 0; j < A.row.size(); ++j)
         m = std::max(m, std::fabs(a) * A.row[i] * B.row[j] + std::fabs(b) * B.row[i] * A.row[j]);
@@ -818,7 +818,7 @@ struct SfPlans {
     const double kx = c->kvec[0], ky = c->kvec[1], kz = c->kvec[2];
     // T: k_y C P + k_z M Q in the scale rho, then y = fC S + fM T in the scale 2^eta
     const long double nM = M.norm, nC = C.norm, tiny = 1e-300;
-    const long double rho = std::max(pair_bound(ky, kz, C, M), tiny);
+    const long double rho = std::max((long double)pair_bound(ky, kz, C, M), tiny);
     const int eta = fx_scale((double)std::max(std::fabs(f) * std::max(std::fabs(kx) * nC * nM * nM, nM * rho), tiny));
     M.put(t.M, 1 / nM);
     C.put(t.C, 1 / nC);
@@ -846,7 +846,7 @@ struct SfPlans {
     const double alpha = t.bad ? 1.0 : alpha_in;
     // scales (see FxLocal); without a kinetic part c is cM / 2 in the scale of cM
     const long double nM = M.norm, nD = D.norm, nP = phi.norm, nS = psi.norm, p3 = nP * nP * nP, akf = std::fabs(kf);
-    t.mf = (double)(mf * nM * nM / (t.hasK ? pair_bound(kf, kf, D, M) * 16 / 15
+    t.mf = (double)(mf * nM * nM / (t.hasK ? (long double)pair_bound(kf, kf, D, M) * 16 / 15
                                            : mf * nM * nM * 2 * std::max(std::fabs(cM) * (1 + 1e-6L), 1e-270L)));
     const long double rho = mf * nM * nM / t.mf;   // c = cM t.mf has no other rounding
     t.eta = fx_scale((double)std::max(std::fabs(alpha) * std::max(akf * nD * nM * nM, nM * rho), tiny));
